@@ -58,7 +58,8 @@ void iteration(const Shape& s, Buffers& b, bool fp64, bool first, cudaStream_t s
   NA_CUDA(launch_apply_v(s, b, fp64, st));
   NA_CUDA(launch_sweep(s, b, fp64, u_new, st));
   NA_CUDA(launch_iter_end(s, b, fp64, st));
-  NA_CUDA(launch_gram_p(s, b, fp64, true, st));
+  NA_CUDA(launch_gram_p(s, b, fp64, true, st, fp64 && !b.plain ? b.U[u_new] : nullptr, fp64 && !b.plain ? b.B : nullptr));
+  b.d_plain = b.plain;
   b.u_cur = u_new;
   std::swap(b.Y[0], b.Y[1]);
 }
@@ -124,6 +125,7 @@ extern "C" sfr_status sfr_solve_noalloc(sfr_ctx* ctx, const sfr_problem* prob, s
     NA_CUDA(cudaMemcpyAsync(b.Qeig_u, eyef, 4 * s.rp * s.rp, cudaMemcpyHostToDevice, st));
     NA_CUDA(cudaMemcpyAsync(b.Qeig_v, eyef, 4 * s.rp * s.rp, cudaMemcpyHostToDevice, st));
     NA_CUDA(launch_norm_m(s, b, st));
+    b.plain = plain_start(s.rp, fp64);
     iteration(s, b, fp64, true, st);
     const Buffers after_first = b;
     DevState out{};
@@ -133,7 +135,10 @@ extern "C" sfr_status sfr_solve_noalloc(sfr_ctx* ctx, const sfr_problem* prob, s
       NA_CUDA(cudaMemcpyAsync(&out, b.st, sizeof out, cudaMemcpyDeviceToHost, st));
       NA_CUDA(cudaStreamSynchronize(st));
       if (out.done || launched >= cap) break;
-      for (int k = 0; k < 8 && launched < cap; ++k, ++launched) iteration(s, b, fp64, false, st);
+      for (int k = 0; k < 8 && launched < cap; ++k, ++launched) {
+        b.plain = plain_start(s.rp, fp64) && launched < kPlainIters;
+        iteration(s, b, fp64, false, st);
+      }
     }
     // buffers of the last completed iteration K: iterations after the first alternate them
     const int K = out.iter;

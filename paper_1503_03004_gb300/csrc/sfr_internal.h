@@ -79,6 +79,7 @@ struct Shape {
   int cols_per_split;   // multiple of the sweep's column tile
   int nchunk;           // row chunks of the W = X^T U pass
   int rows_per_chunk;   // multiple of the W pass's row tile
+  int nchunk64, rows_per_chunk64;  // the same for the float64 path's W pass (at most nchunk chunks)
   int sweep_grid_x;     // ceil(m / sweep rows per CTA)
   int wpass_grid_x;     // ceil(n / W-pass columns per CTA)
   int gram_rows;        // rows per CTA in the Gram / row-transform kernels
@@ -111,7 +112,7 @@ struct Buffers {
   int64_t ldy;          // leading dimension of Y[] and D: n, rounded up to 4 on the SIMT mixed path
                         // (16-byte aligned rows for its vector and cp.async accesses)
   void* Y[2];           // multiplier ping-pong, m x ldy, TC
-  void* D;              // Delta = X_{k+1} - L_{k+1}, m x ldy, TC
+  void* D;              // Delta = X_{k+1} - L_{k+1}, m x ldy, TC (float64 path: fixed point, fix64.cuh)
   void* P;              // m x rp, TC: X_k V_k
   void* U[2];           // m x rp, TC: U_bar ping-pong
   void* W;              // n x rp, TC: X_k^T U_bar
@@ -132,16 +133,29 @@ struct Buffers {
   double* TCm;          // rp x rp : C = W T_C
   float* Qeig_u;        // rp x rp : last U-side eigenvectors (warm start)
   float* Qeig_v;        // rp x rp : last V-side eigenvectors
+  int* ex;              // float64 path: exponents of the fixed-point tiles of U, C and V (64 rows each)
   DevState* st;
   int u_cur;            // which U buffer holds the current U_bar (host-side bookkeeping)
   bool tc;              // tensor-core path (mixed precision, r <= 64, bfloat16 M)
+  bool plain;           // float64 path: this iteration's products are float64 loops (kPlainIters)
+  bool d_plain;         // D holds float64 values (the last sweep was a plain one)
   bool full;            // Algorithm 4 on a fixed M: no multiplier or Delta buffers; the
                         // tensor-core path keeps two-term bfloat16 splits of U^T and V^T
   TcBuffers t;          // its extra buffers (Y[] above alias t.Y[] when tc)
 };
 
-// ---- kernel launchers (sweep.cu / rxr.cu) ----
+// ---- kernel launchers (sweep.cu / rxr.cu / f64.cu) ----
 // Each launcher returns the cudaError_t of its launch.
+
+// Float64 path (f64.cu), behind the launchers of the same names below.  Between apply_v and the
+// next gram_p, P holds U_bar in fixed point, W holds V_bar and the first W partial holds C.
+cudaError_t f64_gram(const Shape& s, const double* parts, int nparts, int64_t part_stride, double* out, int64_t rows,
+                     int ctas, const double* A, const double* H, double* gpart, const DevState* dst, cudaStream_t st);
+cudaError_t f64_transform(const Shape& s, const double* src, int64_t rows, int ctas, const double* T, double* dst,
+                          const double* T2, double* dst2, const double* old, double* hpart, void* F, int* eF, void* F2,
+                          int* eF2, const DevState* dstate, cudaStream_t st);
+cudaError_t f64_sweep(const Shape& s, const Buffers& b, cudaStream_t st);
+cudaError_t f64_wpass(const Shape& s, const Buffers& b, cudaStream_t st);
 
 cudaError_t launch_norm_m(const Shape& s, const Buffers& b, cudaStream_t st);
 cudaError_t launch_init_p(const Shape& s, const Buffers& b, bool fp64, cudaStream_t st);
@@ -178,6 +192,16 @@ constexpr int kSweepBN = 64;     // columns per sweep tile
 constexpr int kWBN = 64;         // columns per W-pass CTA
 constexpr int kWBM = 32;         // rows per W-pass tile
 constexpr int kGramRows = 64;    // rows per Gram / transform CTA
+
+// Float64 solves of rank above 16 run their first iterations with float64 multiply-add loops (sweep.cu's
+// kernels) and switch to the fixed-point products of f64.cu after kPlainIters.  In those iterations the
+// projector starts far from its previous eigenbasis and corrects it in float32: a last-bit change of a
+// Gram matrix then turns U, B and V together by up to 1e-9 (L and S stay within 1e-13), where later it
+// moves them by 1e-14, so keeping the arithmetic of the start keeps the factors reproducible.  Turned
+// by, over 20 inputs each, without a plain start: 2.5e-10 at 500 x 500, r = 25, 6.4e-10 at 300 x 260, r = 32, 1e-9 at 4096 x
+// 4096, r = 64, but 1.4e-11 at r = 10; with it 3e-13 at r = 64.  kPlainIters + 1 is odd: the buffers alternate every iteration.
+constexpr int kPlainIters = 6;
+inline bool plain_start(int rp, bool fp64) { return fp64 && rp > 16; }
 
 inline int pad_rank(int r) { return r <= 8 ? 8 : r <= 16 ? 16 : r <= 32 ? 32 : 64; }
 // The mixed path's float32 SIMT passes for r <= 32 (sweep_mx*/wpass_mx* kernels).

@@ -118,6 +118,19 @@ Shape plan_shape(int64_t m, int64_t n, int64_t ldm, int r, int num_sms) {
   int64_t rtpc = (rtiles + nc - 1) / nc;
   s.rows_per_chunk = (int)(((rtpc * kWBM) + 63) / 64 * 64);
   s.nchunk = (int)((m + s.rows_per_chunk - 1) / s.rows_per_chunk);
+  // float64 W pass (bound by arithmetic): of at most nchunk chunks, the number that leaves the fewest
+  // rows on the SM with the most CTAs (4096 x 4096: 4 chunks, 2 CTAs of 1024 rows on an SM, instead of
+  // 5, 3 of 832 rows)
+  s.nchunk64 = s.nchunk;
+  s.rows_per_chunk64 = s.rows_per_chunk;
+  for (int k = s.nchunk; k >= 1; --k) {
+    const int64_t rows = ((m + k - 1) / k + 63) / 64 * 64, chunks = (m + rows - 1) / rows;
+    auto load = [&](int64_t ch, int64_t rw) { return (s.wpass_grid_x * ch + num_sms - 1) / num_sms * rw; };
+    if (load(chunks, rows) < load(s.nchunk64, s.rows_per_chunk64)) {
+      s.nchunk64 = (int)chunks;
+      s.rows_per_chunk64 = (int)rows;
+    }
+  }
   s.gram_rows = kGramRows;
   // thin kernels loop over 64-row tiles with at most four CTAs per SM (latency hiding for tall
   // matrices), which bounds the number of r x r partials the projector kernels reduce
@@ -178,7 +191,9 @@ size_t carve(const Shape& s, bool fp64, void* base, Buffers* b, bool tc, bool fu
   x.GWpart = static_cast<double*>(c.take(8 * rpsq * s.gw_blocks));
   x.Hpart = static_cast<double*>(c.take(8 * rpsq * (s.gp_blocks + 1)));
   x.Gsum = static_cast<double*>(c.take(8 * rpsq));
-  x.resid_part = static_cast<double*>(c.take(8 * (size_t)s.resid_parts));
+  // (the float64 sweep writes one residual partial per CTA)
+  x.resid_part = static_cast<double*>(c.take(8 * (fp64 && !full ? (size_t)s.sweep_grid_x * s.nsplit : (size_t)s.resid_parts)));
+  if (fp64 && !full) x.ex = static_cast<int*>(c.take(4 * ((s.m + 63) / 64 + 2 * ((s.n + 63) / 64))));
   x.normm_part = static_cast<double*>(c.take(8 * 1024));
   x.B = static_cast<double*>(c.take(8 * rpsq));
   x.Bprev = static_cast<double*>(c.take(8 * rpsq));
@@ -470,7 +485,10 @@ struct Solver {
     SFR_CUDA(launch_apply_v(s, b, fp64, st));                                 // V_bar, C
     timed_launch(slot, 0, [&] { return launch_sweep(s, b, fp64, u_new, st); });  // S/Y steps, Delta, next P
     SFR_CUDA(launch_iter_end(s, b, fp64, st));                                // residual, mu, stop test
-    SFR_CUDA(launch_gram_p(s, b, fp64, true, st));                            // P = sum of partials, G_P
+    // P = sum of partials (float64: of Delta V_bar, + U_bar B_bar, as on the tensor-core path), G_P
+    SFR_CUDA(launch_gram_p(s, b, fp64, true, st, fp64 && !b.plain ? b.U[u_new] : nullptr,
+                           fp64 && !b.plain ? b.B : nullptr));
+    b.d_plain = b.plain;
     kernels += (first ? 11 : 12) + (s.nchunk >= 32 ? 1 : 0);  // as on the tensor-core path below (+ W pre-sum)
     b.u_cur = u_new;
     std::swap(b.Y[0], b.Y[1]);
@@ -533,9 +551,9 @@ struct Solver {
   // next one already runs, so the GPU does not wait for the host; a launch issued after
   // convergence finds the stop flag set and costs only its launches.  `iter(b, slot)` enqueues
   // one iteration (event slot `slot`) and returns its kernel count.  On return host_state holds
-  // the final device state.
+  // the final device state.  `eager` (odd): how many iterations were launched before.
   template <typename F>
-  void drive(const Buffers& after_first, const std::string& key, int cap, bool timed_first, F&& iter) {
+  void drive(const Buffers& after_first, const std::string& key, int cap, bool timed_first, F&& iter, int eager = 1) {
     Buffers b = after_first;
     if (graph_key != key + (profile ? "/p" : "")) {
       for (cudaGraphExec_t* gp : {&graph, &graph_b})
@@ -569,7 +587,7 @@ struct Solver {
     SFR_CUDA(cudaMemcpyAsync(host_state, after_first.st, sizeof(DevState), cudaMemcpyDeviceToHost, stream));
     SFR_CUDA(cudaStreamSynchronize(stream));
     if (timed_first) harvest(0, host_state->iter >= 1 ? 1 : 0);
-    int launched = 1, last_iter = host_state->iter, which = 0;
+    int launched = eager, last_iter = host_state->iter, which = 0;
     int queue[2], queued = 0;  // launched graphs whose state has not been read yet (oldest first)
     bool stop = host_state->done != 0;
     while (!stop) {
@@ -671,17 +689,22 @@ struct Solver {
     if (profile) make_events();
     if (!tc && mx_path(s, fp64)) tune_mx(s, b, p.m_dtype);
 
-    // iteration 1 (X_1 = M, V_1 = I_{n x r}), eager
-    count(SFR_STAT_ALL, enqueue_iteration(s, b, fp64, true, 0));
-    count(SFR_STAT_SWEEP, 1);
-    count(SFR_STAT_WPASS, 1);
-    count(SFR_STAT_RXR, 2);
+    // iteration 1 (X_1 = M, V_1 = I_{n x r}), eager; with a plain start (kPlainIters) also the plain
+    // iterations and the first one after them
+    const int eager = plain_start(s.rp, fp64) ? kPlainIters + 1 : 1;
+    for (int k = 0; k < eager; ++k) {
+      b.plain = eager > 1 && k < kPlainIters;
+      count(SFR_STAT_ALL, enqueue_iteration(s, b, fp64, k == 0, 0));
+    }
+    count(SFR_STAT_SWEEP, eager);
+    count(SFR_STAT_WPASS, eager);
+    count(SFR_STAT_RXR, 2 * eager);
     const Buffers after_first = b;
     const std::string key = fmt("%p/%lld/%lld/%lld/%d/%d/%p", work.ptr, (long long)s.m, (long long)s.n,
                                 (long long)s.ldm, s.r, (int)fp64, Mdev) +
                             fmt("/%d/%d/%d", (int)p.m_dtype, (int)tc, s.mx_grid_x);
     drive(after_first, key, h.max_iter, true,
-          [&](Buffers& bb, int slot) { return enqueue_iteration(s, bb, fp64, false, slot); });
+          [&](Buffers& bb, int slot) { return enqueue_iteration(s, bb, fp64, false, slot); }, eager);
     DevState out = *host_state;
     const int K = out.iter;
     // buffers of the last completed iteration (see the graph's two-iteration period)

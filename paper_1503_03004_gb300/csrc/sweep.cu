@@ -1504,6 +1504,16 @@ cudaError_t by_rank(int rp, F&& f) {
   }
 }
 
+// Padded ranks whose float64 solves start with plain iterations (plain_start).
+template <typename F>
+cudaError_t by_plain_rank(int rp, F&& f) {
+  switch (rp) {
+    case 32: return f(std::integral_constant<int, 32>{});
+    case 64: return f(std::integral_constant<int, 64>{});
+    default: return cudaErrorInvalidValue;
+  }
+}
+
 template <typename F>
 cudaError_t by_mtype(sfr_dtype dt, const void* M, F&& f) {
   switch (dt) {
@@ -1609,40 +1619,57 @@ cudaError_t launch_init_p(const Shape& s, const Buffers& b, bool fp64, cudaStrea
 
 cudaError_t launch_gram_p(const Shape& s, const Buffers& b, bool fp64, bool sum_parts, cudaStream_t st,
                           const void* addA, const double* H, bool pt) {
-  return by_prec(fp64, [&](auto tc) {
-    using TC = decltype(tc);
-    return by_rank(s.rp, [&](auto rpc) {
+  if (fp64 && !b.plain)
+    return f64_gram(s, static_cast<const double*>(b.Qpart), sum_parts ? s.nsplit : 0, s.m * s.rp,
+                    static_cast<double*>(b.P), s.m, s.gp_blocks, static_cast<const double*>(addA), H, b.GPpart, b.st, st);
+  if (fp64)
+    return by_plain_rank(s.rp, [&](auto rpc) {
       constexpr int RP = decltype(rpc)::value;
-      const size_t sm = gram_smem<TC, RP>();
-      launch_k<&thin_gram_body<TC, RP>, 256>(s.gp_blocks, 256, sm, st,
-          static_cast<const TC*>(b.Qpart), sum_parts ? s.nsplit : 0, s.m * RP, static_cast<TC*>(b.P), s.m,
-          static_cast<const TC*>(addA), H, b.GPpart, b.st, s.q_ctas, (s.n + 63) / 64, (const double*)nullptr,
-          pt ? static_cast<__nv_bfloat16*>(b.t.Ut) : nullptr, (int64_t)b.t.ldd);
-      return cudaGetLastError();
+      return launch_k<&thin_gram_body<double, RP>, 256>(s.gp_blocks, 256, gram_smem<double, RP>(), st,
+          static_cast<const double*>(b.Qpart), sum_parts ? s.nsplit : 0, s.m * RP, static_cast<double*>(b.P), s.m,
+          (const double*)nullptr, (const double*)nullptr, b.GPpart, b.st, 0, (int64_t)0, (const double*)nullptr,
+          (__nv_bfloat16*)nullptr, (int64_t)0);
     });
+  return by_rank(s.rp, [&](auto rpc) {
+    constexpr int RP = decltype(rpc)::value;
+    const size_t sm = gram_smem<float, RP>();
+    launch_k<&thin_gram_body<float, RP>, 256>(s.gp_blocks, 256, sm, st,
+        static_cast<const float*>(b.Qpart), sum_parts ? s.nsplit : 0, s.m * RP, static_cast<float*>(b.P), s.m,
+        static_cast<const float*>(addA), H, b.GPpart, b.st, s.q_ctas, (s.n + 63) / 64, (const double*)nullptr,
+        pt ? static_cast<__nv_bfloat16*>(b.t.Ut) : nullptr, (int64_t)b.t.ldd);
+    return cudaGetLastError();
   });
 }
 
 cudaError_t launch_apply_u(const Shape& s, const Buffers& b, bool fp64, bool first, cudaStream_t st) {
   // U_new = P T_U into the other U buffer; H partials U_old^T U_new (iteration >= 2).
   const int u_old = b.u_cur, u_new = 1 - b.u_cur;
-  return by_prec(fp64, [&](auto tc) {
-    using TC = decltype(tc);
-    return by_rank(s.rp, [&](auto rpc) {
+  if (fp64 && b.plain)
+    return by_plain_rank(s.rp, [&](auto rpc) {
       constexpr int RP = decltype(rpc)::value;
-      const size_t sm = transform_smem<TC, RP>();
-      // tensor-core path: also the TF32 split of U_new (the sweep's operand) and, for the first
-      // W pass, its bfloat16 transpose (later W passes take P^T from the P / Gram kernel)
-      // (Algorithm 4: the two-term bfloat16 split of U^T instead, the B operand of M^T U)
-      const bool tcx = b.tc && RP == 64 && !fp64, tf = tcx && !b.full;
-      launch_k<&row_transform_body<TC, RP>, 256>(s.gp_blocks, 256, sm, st,
-          static_cast<const TC*>(b.P), s.m, b.TU, static_cast<TC*>(b.U[u_new]), nullptr, nullptr,
-          first ? nullptr : static_cast<const TC*>(b.U[u_old]), first ? nullptr : b.Hpart, b.st,
-          tf ? b.t.Uh : nullptr, tf ? b.t.Ul : nullptr,
-          (tcx && (first || b.full)) ? static_cast<__nv_bfloat16*>(b.t.Ut) : nullptr, (int64_t)b.t.ldd,
-          b.full ? 1 : 0);
-      return cudaGetLastError();
+      return launch_k<&row_transform_body<double, RP>, 256>(s.gp_blocks, 256, transform_smem<double, RP>(), st,
+          static_cast<const double*>(b.P), s.m, b.TU, static_cast<double*>(b.U[u_new]), (const double*)nullptr,
+          (double*)nullptr, first ? nullptr : static_cast<const double*>(b.U[u_old]), first ? nullptr : b.Hpart, b.st,
+          (float*)nullptr, (float*)nullptr, (__nv_bfloat16*)nullptr, (int64_t)0, 0);
     });
+  if (fp64)
+    return f64_transform(s, static_cast<const double*>(b.P), s.m, s.gp_blocks, b.TU, static_cast<double*>(b.U[u_new]),
+                         nullptr, nullptr, first ? nullptr : static_cast<const double*>(b.U[u_old]),
+                         first ? nullptr : b.Hpart, b.full ? nullptr : b.P, b.ex, nullptr, nullptr, b.st, st);
+  return by_rank(s.rp, [&](auto rpc) {
+    constexpr int RP = decltype(rpc)::value;
+    const size_t sm = transform_smem<float, RP>();
+    // tensor-core path: also the TF32 split of U_new (the sweep's operand) and, for the first
+    // W pass, its bfloat16 transpose (later W passes take P^T from the P / Gram kernel)
+    // (Algorithm 4: the two-term bfloat16 split of U^T instead, the B operand of M^T U)
+    const bool tcx = b.tc && RP == 64, tf = tcx && !b.full;
+    launch_k<&row_transform_body<float, RP>, 256>(s.gp_blocks, 256, sm, st,
+        static_cast<const float*>(b.P), s.m, b.TU, static_cast<float*>(b.U[u_new]), nullptr, nullptr,
+        first ? nullptr : static_cast<const float*>(b.U[u_old]), first ? nullptr : b.Hpart, b.st,
+        tf ? b.t.Uh : nullptr, tf ? b.t.Ul : nullptr,
+        (tcx && (first || b.full)) ? static_cast<__nv_bfloat16*>(b.t.Ut) : nullptr, (int64_t)b.t.ldd,
+        b.full ? 1 : 0);
+    return cudaGetLastError();
   });
 }
 
@@ -1696,9 +1723,14 @@ cudaError_t launch_wpass(const Shape& s, const Buffers& b, bool fp64, bool first
           return cudaGetLastError();
         });
       }
-      launch_pdl(wpass_kernel<TC, TC, RP>, grid, 256, 0, st, static_cast<const TC*>(b.D), s.n, s.m, s.n, s.rows_per_chunk, U, Wp,
-                                                     b.st);
-      return cudaGetLastError();
+      if constexpr (std::is_same<TC, double>::value && RP < 32) {
+        return f64_wpass(s, b, st);
+      } else {
+        if (std::is_same<TC, double>::value && !b.d_plain) return f64_wpass(s, b, st);
+        launch_pdl(wpass_kernel<TC, TC, RP>, grid, 256, 0, st, static_cast<const TC*>(b.D), s.n, s.m, s.n, s.rows_per_chunk,
+                   U, Wp, b.st);
+        return cudaGetLastError();
+      }
     });
   });
 }
@@ -1714,47 +1746,68 @@ cudaError_t launch_wfinal(const Shape& s, const Buffers& b, bool fp64, bool firs
     if (e != cudaSuccess) return e;
   }
   const double* H = b.Hpart + (size_t)s.gp_blocks * s.rp * s.rp;
-  return by_prec(fp64, [&](auto tc) {
-    using TC = decltype(tc);
-    return by_rank(s.rp, [&](auto rpc) {
-      constexpr int RP = decltype(rpc)::value;
-      const size_t sm = gram_smem<TC, RP>();
-      cudaError_t e;
-      // many row chunks over few columns (tall M): sum the chunks' partials into the first one
-      // with a wide reduction first, so the thin kernel does not add hundreds of them per element
-      int nparts = s.nchunk;
-      if (nparts >= 32) {
-        const int64_t len = s.n * RP;
-        launch_k<&reduce_sq_body<TC>, 1024>(cdiv(len, 32), reduce_threads(nparts), 0, st,
-                                            static_cast<const TC*>(b.Wpart), (int64_t)nparts, len,
-                                            static_cast<TC*>(b.Wpart), b.st);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        nparts = 1;
-      }
-      launch_k<&thin_gram_body<TC, RP>, 256>(s.gw_blocks, 256, sm, st,
-          static_cast<const TC*>(b.Wpart), nparts, s.n * RP, static_cast<TC*>(b.W), s.n,
-          first ? nullptr : static_cast<const TC*>(b.C), first ? nullptr : H, b.GWpart, b.st, 0, (int64_t)0,
-          wp ? (const double*)b.TU : (const double*)nullptr, (__nv_bfloat16*)nullptr, (int64_t)0);
+  // many row chunks over few columns (tall M): sum the chunks' partials into the first one
+  // with a wide reduction first, so the thin kernel does not add hundreds of them per element
+  int nparts = fp64 && !first && !b.d_plain ? s.nchunk64 : s.nchunk;
+  if (nparts >= 32) {
+    const int64_t len = s.n * s.rp;
+    cudaError_t e = by_prec(fp64, [&](auto tc) {
+      using TC = decltype(tc);
+      launch_k<&reduce_sq_body<TC>, 1024>(cdiv(len, 32), reduce_threads(nparts), 0, st, static_cast<const TC*>(b.Wpart),
+                                          (int64_t)nparts, len, static_cast<TC*>(b.Wpart), b.st);
       return cudaGetLastError();
     });
+    if (e != cudaSuccess) return e;
+    nparts = 1;
+  }
+  if (fp64 && b.plain)
+    return by_plain_rank(s.rp, [&](auto rpc) {
+      constexpr int RP = decltype(rpc)::value;
+      return launch_k<&thin_gram_body<double, RP>, 256>(s.gw_blocks, 256, gram_smem<double, RP>(), st,
+          static_cast<const double*>(b.Wpart), nparts, s.n * RP, static_cast<double*>(b.W), s.n,
+          first ? nullptr : static_cast<const double*>(b.C), first ? nullptr : H, b.GWpart, b.st, 0, (int64_t)0,
+          (const double*)nullptr, (__nv_bfloat16*)nullptr, (int64_t)0);
+    });
+  if (fp64)
+    return f64_gram(s, static_cast<const double*>(b.Wpart), nparts, s.n * s.rp, static_cast<double*>(b.W), s.n, s.gw_blocks,
+                    first ? nullptr : static_cast<const double*>(b.C), first ? nullptr : H, b.GWpart, b.st, st);
+  return by_rank(s.rp, [&](auto rpc) {
+    constexpr int RP = decltype(rpc)::value;
+    const size_t sm = gram_smem<float, RP>();
+    launch_k<&thin_gram_body<float, RP>, 256>(s.gw_blocks, 256, sm, st,
+        static_cast<const float*>(b.Wpart), nparts, s.n * RP, static_cast<float*>(b.W), s.n,
+        first ? nullptr : static_cast<const float*>(b.C), first ? nullptr : H, b.GWpart, b.st, 0, (int64_t)0,
+        wp ? (const double*)b.TU : (const double*)nullptr, (__nv_bfloat16*)nullptr, (int64_t)0);
+    return cudaGetLastError();
   });
 }
 
 cudaError_t launch_apply_v(const Shape& s, const Buffers& b, bool fp64, cudaStream_t st) {
-  return by_prec(fp64, [&](auto tc) {
-    using TC = decltype(tc);
-    return by_rank(s.rp, [&](auto rpc) {
+  if (fp64 && b.plain)
+    return by_plain_rank(s.rp, [&](auto rpc) {
       constexpr int RP = decltype(rpc)::value;
-      const size_t sm = transform_smem<TC, RP>();
-      // tensor-core path: also the TF32 split of C and the bfloat16 transpose of V
-      // (Algorithm 4: the two-term bfloat16 split of V^T instead, the B operand of M V)
-      const bool tcx = b.tc && RP == 64 && !fp64, tf = tcx && !b.full;
-      launch_k<&row_transform_body<TC, RP>, 256>(s.gw_blocks, 256, sm, st,
-          static_cast<const TC*>(b.W), s.n, b.TV, static_cast<TC*>(b.V), b.TCm, static_cast<TC*>(b.C), nullptr, nullptr,
-          b.st, tf ? b.t.Ch : nullptr, tf ? b.t.Cl : nullptr, tcx ? static_cast<__nv_bfloat16*>(b.t.Vt) : nullptr,
-          (int64_t)b.t.ldy, b.full ? 1 : 0);
-      return cudaGetLastError();
+      return launch_k<&row_transform_body<double, RP>, 256>(s.gw_blocks, 256, transform_smem<double, RP>(), st,
+          static_cast<const double*>(b.W), s.n, b.TV, static_cast<double*>(b.V), b.TCm, static_cast<double*>(b.C),
+          (const double*)nullptr, (double*)nullptr, b.st, (float*)nullptr, (float*)nullptr, (__nv_bfloat16*)nullptr,
+          (int64_t)0, 0);
     });
+  if (fp64) {
+    const int64_t tu = (s.m + kGramRows - 1) / kGramRows, tv = (s.n + kGramRows - 1) / kGramRows;
+    return f64_transform(s, static_cast<const double*>(b.W), s.n, s.gw_blocks, b.TV, static_cast<double*>(b.V), b.TCm,
+                         static_cast<double*>(b.C), nullptr, nullptr, b.full ? nullptr : b.W, b.ex + tu + tv,
+                         b.full ? nullptr : b.Wpart, b.ex + tu, b.st, st);
+  }
+  return by_rank(s.rp, [&](auto rpc) {
+    constexpr int RP = decltype(rpc)::value;
+    const size_t sm = transform_smem<float, RP>();
+    // tensor-core path: also the TF32 split of C and the bfloat16 transpose of V
+    // (Algorithm 4: the two-term bfloat16 split of V^T instead, the B operand of M V)
+    const bool tcx = b.tc && RP == 64, tf = tcx && !b.full;
+    launch_k<&row_transform_body<float, RP>, 256>(s.gw_blocks, 256, sm, st,
+        static_cast<const float*>(b.W), s.n, b.TV, static_cast<float*>(b.V), b.TCm, static_cast<float*>(b.C), nullptr, nullptr,
+        b.st, tf ? b.t.Ch : nullptr, tf ? b.t.Cl : nullptr, tcx ? static_cast<__nv_bfloat16*>(b.t.Vt) : nullptr,
+        (int64_t)b.t.ldy, b.full ? 1 : 0);
+    return cudaGetLastError();
   });
 }
 
@@ -1795,25 +1848,30 @@ static cudaError_t launch_sweep_mx(const Shape& s, const Buffers& b, int u_cur, 
 cudaError_t launch_sweep(const Shape& s, const Buffers& b, bool fp64, int u_cur, cudaStream_t st) {
   // Y ping-pong: iteration k (0-based count of completed iterations) reads Y[k % 2] and writes
   // Y[(k + 1) % 2].  The host tracks k because graphs are replayed per iteration parity.
+  if (fp64 && !b.plain) return f64_sweep(s, b, st);
   if (mx_path(s, fp64)) return launch_sweep_mx(s, b, u_cur, st);
+  // mixed precision above rank 32 outside the tensor-core path, and the plain float64 iterations
   dim3 grid(s.sweep_grid_x, s.nsplit);
   return by_prec(fp64, [&](auto tc) {
     using TC = decltype(tc);
-    return by_rank(s.rp, [&](auto rpc) {
+    return by_plain_rank(s.rp, [&](auto rpc) {
       constexpr int RP = decltype(rpc)::value;
-      const size_t smem = sizeof(TC) * ((size_t)RP * kSweepBM + (size_t)RP * kSweepBN * 2 +
-                                        (size_t)kSweepBM * (kSweepBN + 1));
-      return by_mtype(b.m_dtype, b.M, [&](auto M) {
-        using TMs = std::remove_const_t<std::remove_pointer_t<decltype(M)>>;
-        auto kern = sweep_kernel<TC, TMs, RP>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        launch_pdl(kern, grid, 256, smem, st, M, s.m, s.n, s.ldm, static_cast<const TC*>(b.Y[0]), static_cast<TC*>(b.Y[1]),
-                                      static_cast<TC*>(b.D), static_cast<const TC*>(b.U[u_cur]),
-                                      static_cast<const TC*>(b.C), static_cast<const TC*>(b.V),
-                                      static_cast<TC*>(b.Qpart), s.cols_per_split, b.resid_part, b.st);
-        return cudaGetLastError();
-      });
+      if constexpr (std::is_same<TC, float>::value && RP <= 32) {
+        return cudaErrorInvalidValue;
+      } else {
+        const size_t smem = sizeof(TC) * ((size_t)RP * kSweepBM + (size_t)RP * kSweepBN * 2 +
+                                          (size_t)kSweepBM * (kSweepBN + 1));
+        return by_mtype(b.m_dtype, b.M, [&](auto M) {
+          using TMs = std::remove_const_t<std::remove_pointer_t<decltype(M)>>;
+          auto kern = sweep_kernel<TC, TMs, RP>;
+          cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+          if (e != cudaSuccess) return e;
+          launch_pdl(kern, grid, 256, smem, st, M, s.m, s.n, s.ldm, static_cast<const TC*>(b.Y[0]), static_cast<TC*>(b.Y[1]),
+                     static_cast<TC*>(b.D), static_cast<const TC*>(b.U[u_cur]), static_cast<const TC*>(b.C),
+                     static_cast<const TC*>(b.V), static_cast<TC*>(b.Qpart), s.cols_per_split, b.resid_part, b.st);
+          return cudaGetLastError();
+        });
+      }
     });
   });
 }
