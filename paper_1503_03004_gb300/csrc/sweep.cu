@@ -30,17 +30,22 @@ template <> __device__ __forceinline__ double ld_as<double, __nv_bfloat16>(const
 
 __device__ __forceinline__ bool stopped(const DevState* st) { return *(volatile const int32_t*)&st->done != 0; }
 
-// Block-wide sum of a double; every thread gets the result.  blockDim.x <= 1024.
-// Residual partial of one warp over one row block of a column split of the SIMT mixed sweeps:
-// slot (split, row block, warp), so that the partials (and their fixed-order sum in the
-// iteration end) do not depend on how many CTAs the sweep runs.
-__device__ __forceinline__ void resid_store_warp(float resid, double* __restrict__ resid_part, int64_t split,
-                                                 int64_t nrb, int64_t rb) {
-  double v = (double)resid;
+// Residual partial of one row block of a column split of the SIMT mixed sweeps, from the threads'
+// float32 parts in rs[256] (one warp calls it): slot (split, row block), so that the partials (and
+// their fixed-order sum in the iteration end) do not depend on how many CTAs the sweep runs.  One
+// warp adds all 256 parts in float64: eight warps reducing their own with float64 shuffles took 40
+// float64 operations of the narrow pipe per row block, this takes 12.
+__device__ __forceinline__ void resid_store(const float* rs, double* __restrict__ resid_part, int64_t split, int64_t nrb,
+                                            int64_t rb) {
+  const int lane = threadIdx.x & 31;
+  double v = (double)rs[lane];
+#pragma unroll
+  for (int w = 1; w < 8; ++w) v += (double)rs[lane + 32 * w];
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) resid_part[(split * nrb + rb) * 8 + (threadIdx.x >> 5)] = v;
+  if (lane == 0) resid_part[split * nrb + rb] = v;
 }
 
+// Block-wide sum of a double; every thread gets the result.  blockDim.x <= 1024.
 __device__ double block_sum(double v, double* red) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
@@ -793,7 +798,7 @@ __device__ __forceinline__ void st4(float* __restrict__ p, int lim, const float 
 // 8 tc .. 8 tc + 7 of the tile, loads M and Y_k (vector loads issued before the L products),
 // writes Y_{k+1}, Delta and X = L + Delta (into shared memory).  Phase B: thread (qr, qa) adds
 // X V for rows 2 qr, 2 qr + 1 and ranks qa r/8 .. into registers; the Q partial of a row block is
-// stored once.  One residual partial per (column split, row block, warp) (resid_store_warp).
+// stored once.  One residual partial per (column split, row block) (resid_store).
 template <typename TMs, int RP, bool VEC>
 __device__ __forceinline__ void sweep_mx_body(const VGrid& vg__, const TMs* __restrict__ M, int64_t m, int64_t n, int64_t ldm,
                                                        int64_t ldy, const float* __restrict__ Yin, float* __restrict__ Yout,
@@ -809,6 +814,7 @@ __device__ __forceinline__ void sweep_mx_body(const VGrid& vg__, const TMs* __re
   __shared__ __align__(16) float CsT[RP][BN];
   __shared__ __align__(16) float Vs[BN][RP];
   __shared__ __align__(16) float Xs[BM][kMxLDX];
+  __shared__ float rs[256];
   const double mu_d = st->mu, mu_next = fmin(st->mu_max, st->rho * mu_d);
   const float mu = (float)mu_d, inv_mu = (float)(1.0 / mu_d), dcoef = (float)(1.0 / mu_d + 1.0 / mu_next);
   const int64_t jbeg = (int64_t)blockIdx.y * cols_per_split;
@@ -948,7 +954,9 @@ __device__ __forceinline__ void sweep_mx_body(const VGrid& vg__, const TMs* __re
 #pragma unroll
         for (int k = 0; k < QA; ++k) Qpart[((int64_t)blockIdx.y * m + i) * RP + QA * tc + k] = q[x][k];
     }
-    resid_store_warp(resid, resid_part, blockIdx.y, nrb, rb);
+    rs[t] = resid;
+    __syncthreads();
+    if (t < 32) resid_store(rs, resid_part, blockIdx.y, nrb, rb);
   }
 }
 
@@ -959,90 +967,149 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src, int src_b
                : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 
-// The sweep above with the M and Y_k tiles double-buffered in shared memory by cp.async: the copy
-// of the CTA's next (row block, column tile) pair is in flight while the current one is
-// computed, so HBM latency is hidden without holding the tiles in registers.  Needs the vector
-// conditions (n % 4 == 0, 16-byte aligned rows of M) and float32 or bfloat16 M.
+__device__ __forceinline__ void cp_async4(void* dst, const void* src, int src_bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(src_bytes)
+               : "memory");
+}
+template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+
+// The sweep above with every operand tile brought in by cp.async while earlier tiles are computed.
+// Pair k = the CTA's k-th (row block, column tile).  Y and M stand in a ring of `nst` stages of `tw`
+// columns (64, or n rounded up to 8 for narrow matrices, which leaves room for four stages: at n = 40 two stages kept
+// too few bytes in flight), U in a ring of row blocks, C in two buffers (transposed, its 4-column groups
+// XORed with the rank group, so that neither the 4-byte copies nor the 16-byte reads meet in a bank), V
+// in one, copied while the tile's L is formed.  X = L + Delta overwrites the Y tile.
+// A thread's columns are 4 tc .. + 3 and 32 + 4 tc .. + 3, so that 8 threads read 128 contiguous bytes; sums over
+// ranks and columns run in order, 4 at a time from 16-byte reads (zeros past r and past the last column add nothing).
+// Loading the C and V tiles with plain loads after the barrier (the C stores 32 to a bank) used to take more than
+// half of each tile's time: 4096 x 2048, r = 32, bfloat16: 105 -> 60 us a sweep.
+// Needs the vector conditions (ldy % 4 == 0, 16-byte aligned rows of M) and float32 or bfloat16 M.
 template <typename TMs, int RP>
 __device__ __forceinline__ void sweep_mxp_body(const VGrid& vg__, const TMs* __restrict__ M, int64_t m, int64_t n, int64_t ldm,
                                                         int64_t ldy, const float* __restrict__ Yin, float* __restrict__ Yout,
                                                         float* __restrict__ D, const float* __restrict__ U,
                                                         const float* __restrict__ C, const float* __restrict__ V,
                                                         float* __restrict__ Qpart, int cols_per_split,
-                                                        double* __restrict__ resid_part, int r, const DevState* st) {
+                                                        double* __restrict__ resid_part, int r, int tw, int nst,
+                                                        const DevState* st) {
   pdl_enter();
   SFR_VGRID(vg__);
   if (stopped(st)) return;
   constexpr int BM = kMxBM, BN = kMxBN, QA = RP / 8, EPC = 16 / (int)sizeof(TMs);  // M elements per 16 B
   constexpr int LDU = RP + 4;  // padded U rows: the four rows a warp reads fall in different banks
+  constexpr int QR = RP / 4;   // rank groups
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float* Ys = reinterpret_cast<float*>(smem_raw);                     // [2][BM][BN]
-  TMs* Ms = reinterpret_cast<TMs*>(Ys + 2 * BM * BN);                 // [2][BM][BN]
-  float* Us = reinterpret_cast<float*>(Ms + 2 * BM * BN);             // [2][BM][LDU]: U rows, by row-block parity
-  float* CsT = Us + 2 * BM * LDU;                                     // [RP][BN]
-  float* Vs = CsT + RP * BN;                                          // [BN][RP]
-  float* Xs = Vs + BN * RP;                                           // [BM][kMxLDX]
-  const double mu_d = st->mu, mu_next = fmin(st->mu_max, st->rho * mu_d);
-  const float mu = (float)mu_d, inv_mu = (float)(1.0 / mu_d), dcoef = (float)(1.0 / mu_d + 1.0 / mu_next);
+  __shared__ float rs[256];
+  const int ldx = tw + 4;
   const int64_t jbeg = (int64_t)blockIdx.y * cols_per_split;
   const int64_t jend = min(n, jbeg + cols_per_split);
   const int ntile = (int)((jend - jbeg + BN - 1) / BN);
+  const int nu = ntile == 1 ? nst : 2;
+  float* Ys = reinterpret_cast<float*>(smem_raw);                     // [nst][BM][ldx], then X
+  float* Us = Ys + nst * BM * ldx;                                    // [nu][BM][LDU]
+  float* Cs = Us + (nst > 2 ? nst : 2) * BM * LDU;                    // [2][RP][BN]
+  float* Vs = Cs + 2 * RP * BN;                                       // [BN][RP]
+  TMs* Ms = reinterpret_cast<TMs*>(Vs + BN * RP);                     // [nst][BM][tw]
+  const double mu_d = st->mu, mu_next = fmin(st->mu_max, st->rho * mu_d);
+  const float mu = (float)mu_d, inv_mu = (float)(1.0 / mu_d), dcoef = (float)(1.0 / mu_d + 1.0 / mu_next);
   const int t = threadIdx.x, tr = t >> 3, tc = t & 7;
   const int64_t nrb = (m + BM - 1) / BM;
   const int64_t nmine = blockIdx.x < nrb ? (nrb - 1 - blockIdx.x) / gridDim.x + 1 : 0;
-  const int64_t total = nmine * ntile;  // this CTA's (row block, tile) pairs, row block major
+  const int64_t total = nmine * ntile;
 
-  auto issue = [&](int64_t k) {  // cp.async of pair k into stage k & 1 (and its U rows on tile 0)
-    const int64_t rb = blockIdx.x + (k / ntile) * gridDim.x, i0 = rb * BM;
-    const int64_t j0 = jbeg + (k % ntile) * BN;
-    float* ys = Ys + (k & 1) * BM * BN;
-    TMs* ms = Ms + (k & 1) * BM * BN;
-    if (k % ntile == 0) {
-      float* us = Us + ((k / ntile) & 1) * BM * LDU;
-      for (int e = t; e < BM * (RP / 4); e += blockDim.x) {
-        const int ii = e / (RP / 4), cc = e % (RP / 4);
-        const int64_t i = i0 + ii;
-        cp_async16(us + ii * LDU + 4 * cc, i < m ? (const void*)(U + i * RP + 4 * cc) : (const void*)U, i < m ? 16 : 0);
+  auto issue_v = [&](int64_t j0) {
+    for (int e = t; e < BN * QR; e += 256) {
+      const bool ok = j0 + e / QR < jend;
+      cp_async16(Vs + 4 * e, ok ? (const void*)(V + j0 * RP + 4 * e) : (const void*)V, ok ? 16 : 0);
+    }
+  };
+  // the next pair to copy: row block, column tile, stage, U slot
+  int64_t irb = blockIdx.x;
+  int itile = 0, istage = 0, iu = 0, ic = 0;
+  auto issue = [&] {
+    const int64_t i0 = irb * BM, j0 = jbeg + (int64_t)itile * BN;
+    if (itile == 0) {
+      float* us = Us + iu * BM * LDU;
+      for (int e = t; e < BM * QR; e += 256) {
+        const int ii = e / QR, cc = e % QR;
+        const bool ok = i0 + ii < m;
+        cp_async16(us + ii * LDU + 4 * cc, ok ? (const void*)(U + (i0 + ii) * RP + 4 * cc) : (const void*)U, ok ? 16 : 0);
       }
     }
-    for (int e = t; e < BM * (BN / 4); e += blockDim.x) {  // Y: 16-byte chunks of 4 floats
-      const int ii = e / (BN / 4), cc = e % (BN / 4);
-      const int64_t i = i0 + ii, j = j0 + 4 * cc;
-      const bool ok = i < m && j < jend;
-      cp_async16(ys + ii * BN + 4 * cc, ok ? (const void*)(Yin + i * ldy + j) : (const void*)Yin, ok ? 16 : 0);
+    if (ntile > 1 || ic == 0) {  // C rows j0 + jj, rank 4 q + s -> Cs[4 q + s][jj]
+      float* cs = Cs + (ic & 1) * RP * BN;
+      ++ic;
+#pragma unroll
+      for (int it = 0; it < (RP == 32 ? 8 : 4); ++it) {
+        constexpr int JL = 32 / QR;  // columns a warp covers at a time
+        const int l = t & 31, q = l % QR, sI = it & 3;
+        const int jj = ((it >> 2) * 8 + (t >> 5)) * JL + l / QR, a = 4 * q + sI;
+        if (jj >= BN) continue;
+        const bool ok = j0 + jj < jend;
+        cp_async4(cs + a * BN + (((jj >> 2) ^ q) << 2) + (jj & 3), ok ? (const void*)(C + (j0 + jj) * RP + a) : (const void*)C,
+                  ok ? 4 : 0);
+      }
     }
-    for (int e = t; e < BM * (BN / EPC); e += blockDim.x) {  // M: 16-byte chunks
-      const int ii = e / (BN / EPC), cc = e % (BN / EPC);
-      const int64_t i = i0 + ii, j = j0 + EPC * cc;
-      const int64_t left = i < m ? jend - j : 0;
+    float* ys = Ys + istage * BM * ldx;
+    {
+      const int cc = t & 15;  // 16-byte chunks of a row
+      const bool in = 4 * cc < tw, col = j0 + 4 * cc < jend;
+#pragma unroll
+      for (int it = 0; it < 4; ++it) {
+        const int ii = (t >> 4) + 16 * it;
+        const bool ok = col && i0 + ii < m;
+        if (in) cp_async16(ys + ii * ldx + 4 * cc, ok ? (const void*)(Yin + (i0 + ii) * ldy + j0 + 4 * cc) : (const void*)Yin, ok ? 16 : 0);
+      }
+    }
+    TMs* ms = Ms + istage * BM * tw;
+    {
+      constexpr int CPR = BN / EPC, RPI = 256 / CPR;
+      const int cc = t % CPR;
+      const bool in = EPC * cc < tw;
+      const int64_t left = jend - (j0 + EPC * cc);
       const int bytes = left <= 0 ? 0 : (left >= EPC ? 16 : (int)left * (int)sizeof(TMs));
-      cp_async16(ms + ii * BN + EPC * cc, bytes ? (const void*)(M + i * ldm + j) : (const void*)M, bytes);
+#pragma unroll
+      for (int it = 0; it < BM / RPI; ++it) {
+        const int ii = t / CPR + RPI * it;
+        const bool ok = bytes > 0 && i0 + ii < m;
+        if (in) cp_async16(ms + ii * tw + EPC * cc, ok ? (const void*)(M + (i0 + ii) * ldm + j0 + EPC * cc) : (const void*)M, ok ? bytes : 0);
+      }
     }
-    cp_async_commit();
-  };
-  auto load_cv = [&](int64_t j0) {
-    for (int e = t; e < BN * RP; e += blockDim.x) {
-      const int jj = e / RP, a = e % RP;
-      const int64_t j = j0 + jj;
-      const bool in = j < jend;
-      CsT[a * BN + jj] = in ? C[j * RP + a] : 0.f;
-      Vs[jj * RP + a] = in ? V[j * RP + a] : 0.f;
+    if (++itile == ntile) {
+      itile = 0;
+      irb += gridDim.x;
+      if (++iu == nu) iu = 0;
     }
+    if (++istage == nst) istage = 0;
   };
 
-  if (total > 0) issue(0);
-  if (ntile == 1) load_cv(jbeg);
+  if (ntile == 1 && total > 0) issue_v(jbeg);
+  for (int s = 0; s < nst - 1; ++s) {
+    if (s < total) issue();
+    cp_async_commit();
+  }
   float q[2][QA];
   float resid = 0.f;
+  int64_t rb = blockIdx.x, rb_done = -1;
+  int tile = 0, stage = 0, cu = 0;
   for (int64_t k = 0; k < total; ++k) {
-    const int64_t rb = blockIdx.x + (k / ntile) * gridDim.x, i0 = rb * BM;
-    const int tile = (int)(k % ntile);
-    const int64_t j0 = jbeg + (int64_t)tile * BN;
-    if (k + 1 < total) issue(k + 1); else cp_async_commit();  // keep one group per iteration
-    cp_async_wait1();  // pair k has landed (this thread's copies)
-    __syncthreads();   // everyone's copies visible; the previous pair's Xs / Vs readers are done
+    const int64_t i0 = rb * BM, j0 = jbeg + (int64_t)tile * BN;
+    if (nst == 2) cp_async_wait<0>();  // pair k has landed (this thread's copies)
+    else if (nst == 3) cp_async_wait<1>();
+    else cp_async_wait<2>();
+    __syncthreads();  // everyone's copies visible; the previous pair's readers are done
+    if (rb_done >= 0) {
+      if (t < 32) resid_store(rs, resid_part, blockIdx.y, nrb, rb_done);
+      rb_done = -1;
+    }
+    if (ntile > 1) {
+      issue_v(j0);
+      cp_async_commit();
+    }
+    if (k + nst - 1 < total) issue();
+    cp_async_commit();  // one group per iteration
     if (tile == 0) {
 #pragma unroll
       for (int x = 0; x < 2; ++x)
@@ -1050,102 +1117,107 @@ __device__ __forceinline__ void sweep_mxp_body(const VGrid& vg__, const TMs* __r
         for (int c = 0; c < QA; ++c) q[x][c] = 0.f;
       resid = 0.f;
     }
-    if (ntile > 1) {
-      load_cv(j0);
-      __syncthreads();
-    }
-    const float* us = Us + ((k / ntile) & 1) * BM * LDU;
-    // phase A: L for rows 2 tr, 2 tr + 1 and columns 8 tc .. 8 tc + 7 (ranks a < r)
+    // phase A: L for rows 2 tr, 2 tr + 1 and the thread's two column groups
+    const float* us = Us + cu * BM * LDU + 2 * tr * LDU;
+    const float* cs = Cs + (ntile > 1 ? (int)(k & 1) : 0) * RP * BN;
+    const bool two = tw > 32;
     float l[2][8];
 #pragma unroll
     for (int x = 0; x < 2; ++x)
 #pragma unroll
       for (int c = 0; c < 8; ++c) l[x][c] = 0.f;
-#pragma unroll 4
-    for (int a = 0; a < r; ++a) {
-      const float2 u = make_float2(us[(2 * tr) * LDU + a], us[(2 * tr + 1) * LDU + a]);
-      const float4 c0 = *reinterpret_cast<const float4*>(&CsT[a * BN + 8 * tc]);
-      const float4 c1 = *reinterpret_cast<const float4*>(&CsT[a * BN + 8 * tc + 4]);
-      const float cv[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+#pragma unroll 2
+    for (int a4 = 0; a4 < r; a4 += 4) {
+      const float4 v0 = *reinterpret_cast<const float4*>(us + a4), v1 = *reinterpret_cast<const float4*>(us + LDU + a4);
+      const float u0[4] = {v0.x, v0.y, v0.z, v0.w}, u1[4] = {v1.x, v1.y, v1.z, v1.w};
+      const float* cp = cs + a4 * BN + ((tc ^ ((a4 >> 2) & 7)) << 2);
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        l[0][c] = fmaf(u.x, cv[c], l[0][c]);
-        l[1][c] = fmaf(u.y, cv[c], l[1][c]);
+      for (int s4 = 0; s4 < 4; ++s4) {
+        const float4 c0 = *reinterpret_cast<const float4*>(cp + s4 * BN);
+        l[0][0] = fmaf(u0[s4], c0.x, l[0][0]); l[0][1] = fmaf(u0[s4], c0.y, l[0][1]);
+        l[0][2] = fmaf(u0[s4], c0.z, l[0][2]); l[0][3] = fmaf(u0[s4], c0.w, l[0][3]);
+        l[1][0] = fmaf(u1[s4], c0.x, l[1][0]); l[1][1] = fmaf(u1[s4], c0.y, l[1][1]);
+        l[1][2] = fmaf(u1[s4], c0.z, l[1][2]); l[1][3] = fmaf(u1[s4], c0.w, l[1][3]);
+        if (two) {
+          const float4 c1 = *reinterpret_cast<const float4*>(cp + s4 * BN + 32);
+          l[0][4] = fmaf(u0[s4], c1.x, l[0][4]); l[0][5] = fmaf(u0[s4], c1.y, l[0][5]);
+          l[0][6] = fmaf(u0[s4], c1.z, l[0][6]); l[0][7] = fmaf(u0[s4], c1.w, l[0][7]);
+          l[1][4] = fmaf(u1[s4], c1.x, l[1][4]); l[1][5] = fmaf(u1[s4], c1.y, l[1][5]);
+          l[1][6] = fmaf(u1[s4], c1.z, l[1][6]); l[1][7] = fmaf(u1[s4], c1.w, l[1][7]);
+        }
       }
     }
-    const float* ys = Ys + (k & 1) * BM * BN;
-    const TMs* ms = Ms + (k & 1) * BM * BN;
-    const int64_t jc = j0 + 8 * tc;
-    const int lim = (int)(jend - jc < 8 ? jend - jc : 8);
+    float* ys = Ys + stage * BM * ldx;
+    const TMs* ms = Ms + stage * BM * tw;
 #pragma unroll
-    for (int x = 0; x < 2; ++x) {
-      const int rr = 2 * tr + x;
-      const int64_t i = i0 + rr;
-      float mv[8], yv[8];
-      {
-        const float4 a0 = *reinterpret_cast<const float4*>(ys + rr * BN + 8 * tc);
-        const float4 a1 = *reinterpret_cast<const float4*>(ys + rr * BN + 8 * tc + 4);
-        yv[0] = a0.x; yv[1] = a0.y; yv[2] = a0.z; yv[3] = a0.w; yv[4] = a1.x; yv[5] = a1.y; yv[6] = a1.z; yv[7] = a1.w;
-      }
-      if constexpr (std::is_same<TMs, float>::value) {
-        const float4 a0 = *reinterpret_cast<const float4*>(ms + rr * BN + 8 * tc);
-        const float4 a1 = *reinterpret_cast<const float4*>(ms + rr * BN + 8 * tc + 4);
-        mv[0] = a0.x; mv[1] = a0.y; mv[2] = a0.z; mv[3] = a0.w; mv[4] = a1.x; mv[5] = a1.y; mv[6] = a1.z; mv[7] = a1.w;
-      } else {
-        const uint4 w = *reinterpret_cast<const uint4*>(ms + rr * BN + 8 * tc);
-        const uint32_t wv[4] = {w.x, w.y, w.z, w.w};
+    for (int h = 0; h < 2; ++h) {
+      const int c0 = 32 * h + 4 * tc;
+      if (c0 >= tw) continue;
+      const int64_t jc = j0 + c0;
+      const int lim = (int)(jend - jc < 4 ? jend - jc : 4);  // valid columns (may be <= 0)
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        const int rr = 2 * tr + x;
+        const int64_t i = i0 + rr;
+        const float4 yq = *reinterpret_cast<const float4*>(ys + rr * ldx + c0);
+        const float yv[4] = {yq.x, yq.y, yq.z, yq.w};
+        float mv[4];
+        if constexpr (std::is_same<TMs, float>::value) {
+          const float4 w = *reinterpret_cast<const float4*>(ms + rr * tw + c0);
+          mv[0] = w.x; mv[1] = w.y; mv[2] = w.z; mv[3] = w.w;
+        } else {
+          const uint2 w = *reinterpret_cast<const uint2*>(ms + rr * tw + c0);
+          mv[0] = __uint_as_float(w.x << 16); mv[1] = __uint_as_float(w.x & 0xFFFF0000u);
+          mv[2] = __uint_as_float(w.y << 16); mv[3] = __uint_as_float(w.y & 0xFFFF0000u);
+        }
+        const bool row_ok = i < m;
+        float yn[4], dd[4], xx[4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-          mv[2 * c] = __uint_as_float(wv[c] << 16);
-          mv[2 * c + 1] = __uint_as_float(wv[c] & 0xFFFF0000u);
+          const bool ok = row_ok && c < lim;
+          const float y = yv[c], lv = l[x][4 * h + c];
+          const float z = mv[c] - lv + y * inv_mu;
+          const float y1 = fminf(1.f, fmaxf(-1.f, mu * z));
+          const float d = y1 * dcoef - y * inv_mu;
+          const float dy = y1 - y;
+          resid += ok ? dy * dy : 0.f;
+          yn[c] = y1;
+          dd[c] = d;
+          xx[c] = ok ? lv + d : 0.f;  // X = L + Delta (0 outside the matrix)
+        }
+        *reinterpret_cast<float4*>(ys + rr * ldx + c0) = make_float4(xx[0], xx[1], xx[2], xx[3]);
+        if (row_ok && lim > 0) {
+          *reinterpret_cast<float4*>(Yout + i * ldy + jc) = make_float4(yn[0], yn[1], yn[2], yn[3]);
+          *reinterpret_cast<float4*>(D + i * ldy + jc) = make_float4(dd[0], dd[1], dd[2], dd[3]);
         }
       }
-      const bool row_ok = i < m;
-      float yn[8], dd[8];
-#pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        const bool ok = row_ok && c < lim;
-        const float y = yv[c];
-        const float z = mv[c] - l[x][c] + y * inv_mu;
-        const float y1 = fminf(1.f, fmaxf(-1.f, mu * z));
-        const float d = y1 * dcoef - y * inv_mu;
-        const float dy = y1 - y;
-        resid += ok ? dy * dy : 0.f;
-        yn[c] = y1;
-        dd[c] = d;
-        l[x][c] = ok ? l[x][c] + d : 0.f;  // X = L + Delta (0 outside the matrix)
-      }
-      *reinterpret_cast<float4*>(&Xs[rr * kMxLDX + 8 * tc]) = make_float4(l[x][0], l[x][1], l[x][2], l[x][3]);
-      *reinterpret_cast<float4*>(&Xs[rr * kMxLDX + 8 * tc + 4]) = make_float4(l[x][4], l[x][5], l[x][6], l[x][7]);
-      if (row_ok)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          if (lim <= 4 * h) continue;
-          *reinterpret_cast<float4*>(Yout + i * ldy + jc + 4 * h) =
-              make_float4(yn[4 * h], yn[4 * h + 1], yn[4 * h + 2], yn[4 * h + 3]);
-          *reinterpret_cast<float4*>(D + i * ldy + jc + 4 * h) =
-              make_float4(dd[4 * h], dd[4 * h + 1], dd[4 * h + 2], dd[4 * h + 3]);
-        }
     }
-    __syncthreads();  // Xs complete
+    if (ntile > 1) cp_async_wait<1>();  // V of this tile
+    __syncthreads();                    // X (and V) complete
     const int jn = (int)(jend - j0 < BN ? jend - j0 : BN);  // valid columns of the tile
-#pragma unroll 4
-    for (int jj = 0; jj < jn; ++jj) {
-      const float x0 = Xs[(2 * tr) * kMxLDX + jj], x1 = Xs[(2 * tr + 1) * kMxLDX + jj];
-      float v[QA];
-      if constexpr (QA == 4) {
-        const float4 w = *reinterpret_cast<const float4*>(&Vs[jj * RP + 4 * tc]);
-        v[0] = w.x; v[1] = w.y; v[2] = w.z; v[3] = w.w;
-      } else if constexpr (QA == 2) {
-        const float2 w = *reinterpret_cast<const float2*>(&Vs[jj * RP + 2 * tc]);
-        v[0] = w.x; v[1] = w.y;
-      } else {
-        v[0] = Vs[jj * RP + tc];
-      }
+    const float* x0p = ys + 2 * tr * ldx;
+    const float* vp = Vs + QA * tc;
+#pragma unroll 2
+    for (int jj = 0; jj < jn; jj += 4) {
+      const float4 w0 = *reinterpret_cast<const float4*>(x0p + jj), w1 = *reinterpret_cast<const float4*>(x0p + ldx + jj);
+      const float x0[4] = {w0.x, w0.y, w0.z, w0.w}, x1[4] = {w1.x, w1.y, w1.z, w1.w};
 #pragma unroll
-      for (int c = 0; c < QA; ++c) {
-        q[0][c] = fmaf(x0, v[c], q[0][c]);
-        q[1][c] = fmaf(x1, v[c], q[1][c]);
+      for (int s4 = 0; s4 < 4; ++s4) {
+        float v[QA];
+        if constexpr (QA == 4) {
+          const float4 w = *reinterpret_cast<const float4*>(vp + (jj + s4) * RP);
+          v[0] = w.x; v[1] = w.y; v[2] = w.z; v[3] = w.w;
+        } else if constexpr (QA == 2) {
+          const float2 w = *reinterpret_cast<const float2*>(vp + (jj + s4) * RP);
+          v[0] = w.x; v[1] = w.y;
+        } else {
+          v[0] = vp[(jj + s4) * RP];
+        }
+#pragma unroll
+        for (int c = 0; c < QA; ++c) {
+          q[0][c] = fmaf(x0[s4], v[c], q[0][c]);
+          q[1][c] = fmaf(x1[s4], v[c], q[1][c]);
+        }
       }
     }
     if (tile == ntile - 1) {  // row block done: its Q partial and residual
@@ -1156,16 +1228,25 @@ __device__ __forceinline__ void sweep_mxp_body(const VGrid& vg__, const TMs* __r
 #pragma unroll
           for (int c = 0; c < QA; ++c) Qpart[((int64_t)blockIdx.y * m + i) * RP + QA * tc + c] = q[x][c];
       }
-      resid_store_warp(resid, resid_part, blockIdx.y, nrb, rb);
+      rs[t] = resid;  // summed after the next barrier
+      rb_done = rb;
     }
+    if (++tile == ntile) {
+      tile = 0;
+      rb += gridDim.x;
+      if (++cu == nu) cu = 0;
+    }
+    if (++stage == nst) stage = 0;
   }
-  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  cp_async_wait<0>();
+  __syncthreads();
+  if (rb_done >= 0 && t < 32) resid_store(rs, resid_part, blockIdx.y, nrb, rb_done);
 }
 
 template <typename TMs, int RP>
-constexpr size_t mxp_smem() {
-  return (size_t)2 * kMxBM * kMxBN * (4 + sizeof(TMs)) + (size_t)2 * kMxBM * (RP + 4) * 4 +
-         (size_t)RP * 2 * kMxBN * 4 + (size_t)kMxBM * kMxLDX * 4;
+constexpr size_t mxp_smem(int tw, int nst) {
+  return (size_t)nst * kMxBM * ((tw + 4) * 4 + tw * sizeof(TMs)) + (size_t)(nst > 2 ? nst : 2) * kMxBM * (RP + 4) * 4 +
+         (size_t)RP * 3 * kMxBN * 4;
 }
 
 // W pass, float32: Wpart[c][j][:] = sum over the rows i of chunk c of src[i][j] U[i][:].  CTA:
@@ -1831,12 +1912,19 @@ static cudaError_t launch_sweep_mx(const Shape& s, const Buffers& b, int u_cur, 
         };
         if constexpr (!std::is_same<TMs, double>::value) {
           if (vec) {
-            constexpr size_t sm = mxp_smem<TMs, RP>();
+            // narrow matrices: as many columns as needed and up to four stages in half an SM's shared memory
+            // (grouped launches keep one shape, so that problems of different widths share a launch)
+            int tw = 64, nst = 2;
+            if (!g_recorder && s.n <= 64) {
+              tw = (int)(s.n + 7) / 8 * 8;
+              while (nst < 4 && mxp_smem<TMs, RP>(tw, nst + 1) <= 110 * 1024) ++nst;
+            }
+            const size_t sm = mxp_smem<TMs, RP>(tw, nst);
             return launch_k<&sweep_mxp_body<TMs, RP>, 256>(
                 grid, 256, sm, st, M, s.m, s.n, s.ldm, b.ldy, static_cast<const float*>(b.Y[0]), static_cast<float*>(b.Y[1]),
                 static_cast<float*>(b.D), static_cast<const float*>(b.U[u_cur]), static_cast<const float*>(b.C),
                 static_cast<const float*>(b.V), static_cast<float*>(b.Qpart), s.cols_per_split, b.resid_part, s.r,
-                b.st);
+                tw, nst, b.st);
           }
         }
         return vec ? go(BodyTag<&sweep_mx_body<TMs, RP, true>>{}) : go(BodyTag<&sweep_mx_body<TMs, RP, false>>{});
@@ -1877,9 +1965,9 @@ cudaError_t launch_sweep(const Shape& s, const Buffers& b, bool fp64, int u_cur,
 }
 
 cudaError_t launch_iter_end(const Shape& s, const Buffers& b, bool fp64, cudaStream_t st) {
-  // the mixed SIMT sweep writes one residual partial per (column split, 64-row block, warp), the
+  // the mixed SIMT sweep writes one residual partial per (column split, 64-row block), the
   // float64 SIMT sweep one per 32-row block and split, the tensor-core sweep one per CTA
-  const int count = mx_path(s, fp64) ? s.nsplit * (int)((s.m + 63) / 64) * 8
+  const int count = mx_path(s, fp64) ? s.nsplit * (int)((s.m + 63) / 64)
                                      : (b.tc ? s.resid_parts : s.sweep_grid_x * s.nsplit);
   launch_k<&iter_end_body, 1024>(1, 1024, 0, st, b.resid_part, count, b.st);
   return cudaGetLastError();
