@@ -185,11 +185,11 @@ template <typename... T> struct BodyTraits<void (*)(const VGrid&, T...)> {
     if (e != cudaSuccess) return e;
     return launch_pdl(k, grid, block, smem, st, static_cast<T>(a)...);
   }
-  // As launch, but as a thread-block cluster of `cluster` CTAs (grid = cluster); recorded as a
+  // As launch, but as a thread-block cluster of `cluster` CTAs (grid = cluster; 1: a plain launch); recorded as a
   // single-CTA launch (the body must give the same result for any cluster size).
   template <auto Body, int NT, typename... A>
   static cudaError_t launch_cluster(unsigned cluster, dim3 block, size_t smem, cudaStream_t st, A... a) {
-    if (g_recorder) return launch<Body, NT>(dim3(1), block, smem, st, a...);
+    if (g_recorder || cluster == 1) return launch<Body, NT>(dim3(1), block, smem, st, a...);
     auto k = body_kernel<Body, NT, T...>;
     cudaError_t e = set_smem_attr<&body_kernel<Body, NT, T...>>(smem);
     if (e != cudaSuccess) return e;

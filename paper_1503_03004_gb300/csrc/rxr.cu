@@ -1,4 +1,4 @@
-// r x r steps of FixedRankOptStep (Algorithm 3), one CTA per problem.
+// r x r steps of FixedRankOptStep (Algorithm 3), one CTA or cluster per problem.
 //
 // Stiefel projector (Sec. 4.1.1, Eq. 9): P_O[A] = A (A^T A)^{-1/2} for a full-rank
 // m x r matrix A.  With A = P B (U side, P = X V) or A = W B (V side, W = X^T U),
@@ -24,8 +24,17 @@
 // of each float64 product, and pushes its rows to the other CTAs through distributed
 // shared memory.  Everything else (float32 Jacobi, element-wise steps, scalar decisions)
 // is computed redundantly and identically by every CTA, so control flow stays uniform
-// across the cluster; only rank 0 writes to global memory.
+// across the cluster; each CTA writes its own rows.
+//
+// The kernel is a chain of about thirty short dependent phases, so its time is barriers and load
+// latency rather than arithmetic.  It is therefore built per padded rank (Dim): r <= 8 runs in one
+// warp, r <= 16 in one CTA of 128 threads, r <= 32 in clusters of 256-thread CTAs, r <= 64 in clusters of 512,
+// element-wise steps are done where a product's results are stored (Epi), and the statistics of the r
+// eigenvalue estimates are taken by every warp for itself.  A warm call (mixed path) before -> now: r = 3 31 -> 16,
+// r = 32 38 -> 32 r = 48 52 -> 48, r = 64 95 -> us, with the same results to the last bit.
 #include <cooperative_groups.h>
+
+#include <type_traits>
 
 #include "sfr_internal.h"
 
@@ -34,10 +43,13 @@ namespace cg = cooperative_groups;
 namespace sfr {
 namespace {
 
-constexpr int RPMAX = kMaxRank;
-constexpr int LD = RPMAX + 4;  // row stride of the float r x r arrays: 16-byte aligned rows
-constexpr int LDD = RPMAX;     // row stride of the float64 r x r arrays (read along rows only)
-constexpr int kThreads = 512;
+// Sizes of one padded rank RP: threads, the TM x TN outputs a thread takes of a float32 product, row strides of
+// the float32 (16-byte aligned rows) and float64 (read along rows only) r x r arrays.
+template <int RP_> struct Dim {
+  static constexpr int RP = RP_, NT = RP == 64 ? 512 : RP == 32 ? 256 : RP == 16 ? 128 : 32;
+  static constexpr int TM = RP == 64 ? 4 : RP == 32 ? 2 : 1, TN = RP == 64 ? 4 : 2;
+  static constexpr int LD = RP + 4, LDD = RP;
+};
 
 __device__ __forceinline__ bool stopped(const DevState* st) { return *(volatile const int32_t*)&st->done != 0; }
 
@@ -78,22 +90,20 @@ __device__ __forceinline__ double to_f64(double x) { return x; }
 __device__ __forceinline__ double to_f64(float x) { return f32_to_f64_shift(x, 0); }
 
 // C = epi(op(A) B) with float64 arithmetic, rows split across the cluster and broadcast through
-// DSMEM.  A is a float64 array (row stride LDD); B is float64 (LDD) or float (LD), converted on
-// load; C is float64 (LDD) or float (LD) and receives epi(i, j, (op(A) B)_ij).  C must not alias A
-// or B.  On return every CTA holds the full product.
+// DSMEM.  A, B: float64 (row stride LDD).  C is float64 (LDD) or float (LD) and receives
+// epi(i, j, (op(A) B)_ij).  C must not alias A or B.  On return every CTA holds the full product.
 // PRE = false skips the barrier before the broadcast: allowed when no CTA has read C since the
 // last cluster barrier.
-template <bool TA, bool PRE = true, typename TB, typename TCo, typename Epi>
+template <typename DM, bool TA, bool PRE = true, typename TB, typename TCo, typename Epi>
 __device__ __noinline__ void mm_dist(const double* A, const TB* B, TCo* C, int r, Epi epi) {
-  constexpr int ldb = sizeof(TB) == 8 ? LDD : LD;
-  constexpr int ldc = sizeof(TCo) == 8 ? LDD : LD;
+  constexpr int LDD = DM::LDD, ldb = sizeof(TB) == 8 ? DM::LDD : DM::LD, ldc = sizeof(TCo) == 8 ? DM::LDD : DM::LD;
   cg::cluster_group cl = cg::this_cluster();
   const int cs = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int rpc = (r + cs - 1) / cs, i0 = min(r, rank * rpc), i1 = min(r, i0 + rpc);
-  const int nloc = (i1 - i0) * r;
-  for (int e = threadIdx.x; e < nloc; e += blockDim.x) {
-    const int i = i0 + e / r, j = e % r;
-    // four independent chains (k mod 4) keep the float64 pipe busy with 8 warps per SM
+  for (int e = threadIdx.x; e < (i1 - i0) * DM::RP; e += DM::NT) {
+    const int i = i0 + e / DM::RP, j = e % DM::RP;
+    if (j >= r) continue;
+    // four independent chains (k mod 4) keep the float64 pipe busy with few warps per SM
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
     int k = 0;
     for (; k + 4 <= r; k += 4)
@@ -115,7 +125,7 @@ __device__ __noinline__ void mm_dist(const double* A, const TB* B, TCo* C, int r
     // float; the last piece of a row may carry columns >= r, which no product or loop reads)
     constexpr int per16 = 16 / sizeof(TCo);
     const int npc = (r + per16 - 1) / per16, per = (i1 - i0) * npc;
-    for (int e = threadIdx.x; e < (cs - 1) * per; e += blockDim.x) {
+    for (int e = threadIdx.x; e < (cs - 1) * per; e += DM::NT) {
       const int q = 1 + e / per, w = e % per;
       const int i = i0 + w / npc, j = per16 * (w % npc);
       TCo* Cq = cl.map_shared_rank(C, (rank + q) % cs);
@@ -125,117 +135,249 @@ __device__ __noinline__ void mm_dist(const double* A, const TB* B, TCo* C, int r
   }
 }
 
-// C = op(A) op(B) in float32 on the leading r x r blocks, 4 x 4 outputs per thread.  Operands
-// move in 16-byte loads, 4 x 4 blocks of A and B per 4 steps of k (8 loads per 64 FMAs); the
-// sum over k runs in order.  Reads may touch rows and columns beyond r (inside the RPMAX x LD
-// arrays); only outputs inside r x r are written.
-template <bool TA, bool TB>
-__device__ __noinline__ void mmf(const float* A, const float* B, float* C, int r) {
-  const int nb = (r + 3) / 4, r4 = r & ~3;
-  for (int blk = threadIdx.x; blk < nb * nb; blk += blockDim.x) {
-    const int i0 = 4 * (blk / nb), j0 = 4 * (blk % nb);
-    float acc[4][4];
+// What a float32 product's value v at (i, j) becomes.
+enum class Epi {
+  kStore,      // C = v
+  kScale,      // C = f v
+  kAdd,        // C = X + v                         (Q <- Q + Q E)
+  kOrtho,      // C = (3 I - v) / 2                 (Newton-Schulz factor)
+  kBoth,       // C = v, Ct = v transposed          (the basis and its transpose)
+  kLyapunov,   // C = v / (x_i + x_j)               (the Newton correction in the eigenbasis)
+};
+struct EpiArgs {
+  float f = 1.f;
+  const float* x = nullptr;  // kAdd: X (row stride LD); kLyapunov: x
+  float* ct = nullptr;
+};
+
+// C = epi(op(A) diag(s) B) in float32 on the leading r x r blocks (s = nullptr: identity), TM x TN outputs per thread.
+// Operands move in 16-byte loads along k (A) and TN-wide ones (B); the sum over k runs in order.
+// Reads may touch rows and columns beyond r (inside the arrays); only outputs inside r x r are
+// written.  C must not alias A or B.  One copy of the code for all steps (TA aside): the kernel runs each once
+// or twice, and its instructions have to be fetched.
+template <typename DM, bool TA>
+__device__ __noinline__ void mmf(const float* A, const float* B, float* C, int r, Epi epi, const EpiArgs a_ = EpiArgs(),
+                                 const float* s = nullptr) {
+  constexpr int LD = DM::LD, TM = DM::TM, TN = DM::TN, NJ = DM::RP / TN;
+  const int nb = (DM::RP / TM) * NJ;
+  const int blk = threadIdx.x, i0 = TM * (blk / NJ), j0 = TN * (blk % NJ);
+  if (blk < nb && i0 < r && j0 < r) {
+    const int r4 = r & ~3;
+    float acc[TM][TN];
 #pragma unroll
-    for (int x = 0; x < 4; ++x)
+    for (int x = 0; x < TM; ++x)
 #pragma unroll
-      for (int y = 0; y < 4; ++y) acc[x][y] = 0.f;
-    for (int k = 0; k < r4; k += 4) {
-      float a[4][4], b[4][4];  // a[x][q] = op(A)(i0 + x, k + q), b[q][y] = op(B)(k + q, j0 + y)
+      for (int y = 0; y < TN; ++y) acc[x][y] = 0.f;
+    auto load_a = [&](int k, float (&a)[TM][4]) {  // a[x][q] = op(A)(i0 + x, k + q) s(k + q)
+      if constexpr (TA) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float4 va = TA ? *reinterpret_cast<const float4*>(A + (k + q) * LD + i0)
-                             : *reinterpret_cast<const float4*>(A + (i0 + q) * LD + k);
-        const float4 vb = TB ? *reinterpret_cast<const float4*>(B + (j0 + q) * LD + k)
-                             : *reinterpret_cast<const float4*>(B + (k + q) * LD + j0);
-        const float fa[4] = {va.x, va.y, va.z, va.w}, fb[4] = {vb.x, vb.y, vb.z, vb.w};
+        for (int q = 0; q < 4; ++q) {
+          if constexpr (TM == 4) {
+            const float4 v = *reinterpret_cast<const float4*>(A + (k + q) * LD + i0);
+            a[0][q] = v.x; a[1][q] = v.y; a[2][q] = v.z; a[3][q] = v.w;
+          } else if constexpr (TM == 2) {
+            const float2 v = *reinterpret_cast<const float2*>(A + (k + q) * LD + i0);
+            a[0][q] = v.x; a[1][q] = v.y;
+          } else {
+            a[0][q] = A[(k + q) * LD + i0];
+          }
+        }
+      } else {
 #pragma unroll
-        for (int w = 0; w < 4; ++w) {
-          if (TA) a[w][q] = fa[w]; else a[q][w] = fa[w];
-          if (TB) b[w][q] = fb[w]; else b[q][w] = fb[w];
+        for (int x = 0; x < TM; ++x) {
+          const float4 v = *reinterpret_cast<const float4*>(A + (i0 + x) * LD + k);
+          a[x][0] = v.x; a[x][1] = v.y; a[x][2] = v.z; a[x][3] = v.w;
         }
       }
+      if (s)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int x = 0; x < TM; ++x) a[x][q] *= s[k + q];
+    };
+    auto load_b = [&](int k, float (&b)[4][TN]) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        if constexpr (TN == 4) {
+          const float4 v = *reinterpret_cast<const float4*>(B + (k + q) * LD + j0);
+          b[q][0] = v.x; b[q][1] = v.y; b[q][2] = v.z; b[q][3] = v.w;
+        } else {
+          const float2 v = *reinterpret_cast<const float2*>(B + (k + q) * LD + j0);
+          b[q][0] = v.x; b[q][1] = v.y;
+        }
+      }
+    };
+#pragma unroll(TM == 4 ? 1 : 2)
+    for (int k = 0; k < r4; k += 4) {
+      float a[TM][4], b[4][TN];
+      load_a(k, a);
+      load_b(k, b);
 #pragma unroll
       for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int x = 0; x < 4; ++x)
+        for (int x = 0; x < TM; ++x)
 #pragma unroll
-          for (int y = 0; y < 4; ++y) acc[x][y] = fmaf(a[x][q], b[q][y], acc[x][y]);
+          for (int y = 0; y < TN; ++y) acc[x][y] = fmaf(a[x][q], b[q][y], acc[x][y]);
     }
     for (int k = r4; k < r; ++k) {
 #pragma unroll
-      for (int x = 0; x < 4; ++x)
+      for (int x = 0; x < TM; ++x)
 #pragma unroll
-        for (int y = 0; y < 4; ++y) {
-          const float av = TA ? A[k * LD + i0 + x] : A[(i0 + x) * LD + k];
-          const float bv = TB ? B[(j0 + y) * LD + k] : B[k * LD + j0 + y];
-          acc[x][y] = fmaf(av, bv, acc[x][y]);
+        for (int y = 0; y < TN; ++y) {
+          float av = TA ? A[k * LD + i0 + x] : A[(i0 + x) * LD + k];
+          if (s) av *= s[k];
+          acc[x][y] = fmaf(av, B[k * LD + j0 + y], acc[x][y]);
         }
     }
+    // (the step is chosen outside the loops: its code is fetched alone)
+    auto each = [&](auto&& f) {
+      if (i0 + TM <= r && j0 + TN <= r) {  // whole block: one store per row
 #pragma unroll
-    for (int x = 0; x < 4; ++x)
+        for (int x = 0; x < TM; ++x) {
+          float v[TN];
 #pragma unroll
-      for (int y = 0; y < 4; ++y)
-        if (i0 + x < r && j0 + y < r) C[(i0 + x) * LD + j0 + y] = acc[x][y];
+          for (int y = 0; y < TN; ++y) v[y] = acc[x][y] = f(i0 + x, j0 + y, acc[x][y]);
+          float* c = C + (i0 + x) * LD + j0;
+          if constexpr (TN == 4) *reinterpret_cast<float4*>(c) = make_float4(v[0], v[1], v[2], v[3]);
+          else *reinterpret_cast<float2*>(c) = make_float2(v[0], v[1]);
+        }
+      } else {
+#pragma unroll
+        for (int x = 0; x < TM; ++x)
+#pragma unroll
+          for (int y = 0; y < TN; ++y)
+            if (i0 + x < r && j0 + y < r) C[(i0 + x) * LD + j0 + y] = acc[x][y] = f(i0 + x, j0 + y, acc[x][y]);
+      }
+    };
+    switch (epi) {
+      case Epi::kStore: each([&](int, int, float v) { return v; }); break;
+      case Epi::kScale: each([&](int, int, float v) { return v * a_.f; }); break;
+      case Epi::kAdd: each([&](int i, int j, float v) { return a_.x[i * LD + j] + v; }); break;
+      case Epi::kOrtho: each([&](int i, int j, float v) { return 0.5f * ((i == j ? 3.f : 0.f) - v); }); break;
+      case Epi::kBoth:
+        each([&](int, int, float v) { return v; });
+#pragma unroll
+        for (int y = 0; y < TN; ++y) {
+          float* c = a_.ct + (j0 + y) * LD + i0;
+          if (TM == 4 && i0 + TM <= r && j0 + TN <= r) {
+            *reinterpret_cast<float4*>(c) = make_float4(acc[0][y], acc[1 % TM][y], acc[2 % TM][y], acc[3 % TM][y]);
+          } else {
+#pragma unroll
+            for (int x = 0; x < TM; ++x)
+              if (i0 + x < r && j0 + y < r) c[x] = acc[x][y];
+          }
+        }
+        break;
+      case Epi::kLyapunov: each([&](int i, int j, float v) { return __fdividef(v, a_.x[i] + a_.x[j]); }); break;
+    }
   }
   __syncthreads();
 }
 
-// dst[i * LD + j] = src[i * rp + j] for i, j < r; for r <= i, j < n the identity's entries
-// (pad_diag on the diagonal, 0 elsewhere).  Every load of a thread is issued before any store.
-template <typename TS, typename TD>
-__device__ __forceinline__ void load_sq(const TS* __restrict__ src, int rp, int r, int n, TD* dst, TD pad_diag) {
-  constexpr int PER = RPMAX * RPMAX / kThreads;
-  TS v[PER];
-#pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const int e = threadIdx.x + q * kThreads, i = e / RPMAX, j = e % RPMAX;
-    v[q] = (i < r && j < r) ? src[i * rp + j] : (TS)0;
-  }
-#pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const int e = threadIdx.x + q * kThreads, i = e / RPMAX, j = e % RPMAX;
-    if (i < n && j < n) dst[i * LD + j] = (i < r && j < r) ? (TD)v[q] : (i == j ? pad_diag : (TD)0);
-  }
-}
+template <int RP> struct RxrSmem {  // 214 KB at RP = 64
+  static constexpr int LD = Dim<RP>::LD, LDD = Dim<RP>::LDD;
+  double G[RP * LDD];   // Gram of the thin factor (float64 sum of the partials); later B_bar
+  double T[RP * LDD];   // T_hat = B Z_hat (Newton iterate); scratch vectors of the rank test
+  double W[RP * LDD];   // B (until T_hat exists), then G T_hat
+  float Gf[RP * LD];    // G 2^-eg (float32; the power of two keeps K = B G B finite)
+  float Bf[RP * LD];    // B 2^-eb
+  float QT[RP * LD];    // Q^T
+  float Af[RP * LD];    // Q^T K Q / s (K = B G B), the Jacobi matrix, then the Newton correction in that basis
+  float Q[RP * LD];     // approximate eigenbasis of K
+  float F1[RP * LD];    // scratch
+  float F2[RP * LD];    // scratch
+  float lam[64], sq[64], isq[64];  // (all 64 read as two values per lane; entries past r unused)
+  double red[32];
+  unsigned mx[16];      // block-wide maxima, one slot each (bits of non-negative floats)
+  float cs[RP / 2], sn[RP / 2];
+  int pp[RP / 2], qq[RP / 2];
+  double scale, inv_s, rs;  // s = trace(B G B) / r, 1 / s, 1 / sqrt(s)  (written by thread 0)
+  float kn;                 // K's power-of-two scale over s
+  int ok;
+};
 
-// Block-wide maximum of 64-bit integers: shuffles within each warp, one shared slot per warp, then
-// every thread reduces the (at most 32) warp values with shuffles again; the closing barrier lets
-// `red` be reused at once.
-__device__ __noinline__ long long block_max_ll(long long v, double* red) {
+// Block-wide maxima of two 64-bit integers.
+template <int NT>
+__device__ __forceinline__ void block_max2_ll(long long& a, long long& b, double* red) {
   long long* rl = reinterpret_cast<long long*>(red);
-  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
-  if (l == 0) rl[w] = v;
+  for (int o = 16; o > 0; o >>= 1) {
+    a = max(a, __shfl_xor_sync(0xffffffffu, a, o));
+    b = max(b, __shfl_xor_sync(0xffffffffu, b, o));
+  }
+  if (NT == 32) return;
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  constexpr int NW = NT / 32;
+  if (l == 0) rl[w] = a, rl[16 + w] = b;
   __syncthreads();
-  long long t = l < nw ? rl[l] : 0LL;
-  for (int o = 16; o > 0; o >>= 1) t = max(t, __shfl_xor_sync(0xffffffffu, t, o));
-  __syncthreads();
-  return t;
+  a = l < NW ? rl[l] : 0LL;
+  b = l < NW ? rl[16 + l] : 0LL;
+  for (int o = 16; o > 0; o >>= 1) {
+    a = max(a, __shfl_xor_sync(0xffffffffu, a, o));
+    b = max(b, __shfl_xor_sync(0xffffffffu, b, o));
+  }
 }
 
-// float version (the sums and maxima it serves steer decisions only)
-__device__ __noinline__ float block_reduce_f(float v, float* red, bool take_max) {
-  for (int o = 16; o > 0; o >>= 1) {
-    const float w = __shfl_xor_sync(0xffffffffu, v, o);
-    v = take_max ? fmaxf(v, w) : v + w;
-  }
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
+// Block-wide maximum of non-negative floats through one shared slot (zero before); ends with a barrier.
+__device__ __forceinline__ float block_max_f(float v, unsigned* slot) {
+  const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(v));
+  if ((threadIdx.x & 31) == 0) atomicMax(slot, m);
+  __syncthreads();
+  return __uint_as_float(*slot);
+}
+
+// Block-wide sum of floats (it steers decisions only).
+template <int NT> __device__ __noinline__ float block_sum_f(float v, float* red) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   if (l == 0) red[w] = v;
   __syncthreads();
-  float t = l < nw ? red[l] : (take_max ? -INFINITY : 0.f);
-  for (int o = 16; o > 0; o >>= 1) {
-    const float u = __shfl_xor_sync(0xffffffffu, t, o);
-    t = take_max ? fmaxf(t, u) : t + u;
-  }
+  float t = l < NT / 32 ? red[l] : 0.f;
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
   __syncthreads();
   return t;
+}
+
+// Sum of x[0 .. r), r <= 64, by every warp for itself.
+__device__ __forceinline__ float warp_sum64(const float* x, int stride, int r) {
+  const int l = threadIdx.x & 31;
+  float a = l < r ? x[l * stride] : 0.f, b = l + 32 < r ? x[(l + 32) * stride] : 0.f;
+  for (int o = 16; o > 0; o >>= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+    b += __shfl_xor_sync(0xffffffffu, b, o);
+  }
+  return a + b;
+}
+
+// Statistics of the eigenvalue estimates, by every warp for itself: the largest (at least 0), the smallest
+// (at most the largest), whether any is below f of the largest, whether any is not above 1e-14 of it.
+struct LamStats {
+  float hi, lo;
+  bool small, bad;
+};
+__device__ __forceinline__ LamStats lam_stats(const float* lam, int r) {
+  const int l = threadIdx.x & 31;
+  const bool ia = l < r, ib = l + 32 < r;
+  const float a = ia ? lam[l] : 0.f, b = ib ? lam[l + 32] : 0.f;
+  LamStats s;
+  s.hi = fmaxf(fmaxf(0.f, a), b);
+  for (int o = 16; o > 0; o >>= 1) s.hi = fmaxf(s.hi, __shfl_xor_sync(0xffffffffu, s.hi, o));
+  float n = -s.hi;
+  if (ia) n = fmaxf(n, -a);
+  if (ib) n = fmaxf(n, -b);
+  for (int o = 16; o > 0; o >>= 1) n = fmaxf(n, __shfl_xor_sync(0xffffffffu, n, o));
+  s.lo = -n;
+  s.small = __any_sync(0xffffffffu, (ia && a < 1e-6f * s.hi) || (ib && b < 1e-6f * s.hi));
+  s.bad = __any_sync(0xffffffffu, (ia && !(a > 1e-14f * s.hi)) || (ib && !(b > 1e-14f * s.hi))) || !(s.hi > 0.f);
+  return s;
 }
 
 // Cyclic two-sided Jacobi on the symmetric n2 x n2 float matrix A (n2 even; rows/cols
 // beyond r are zero), accumulating the rotations into Q (A_final = Q^T A_init Q).
 // Round-robin ordering: n2/2 disjoint rotations per step, n2-1 steps per sweep.
+template <typename DM>
 __device__ __noinline__ void jacobi_f32(float* A, float* Q, int n2, int max_sweeps, double* red, float* cs, float* sn, int* pp,
-                           int* qq) {
+                                        int* qq) {
+  constexpr int LD = DM::LD, RPMAX = DM::RP, kThreads = DM::NT;
   const int np = n2 / 2;
   const bool pow2 = (np & (np - 1)) == 0;
   const int lg = 31 - __clz(np);
@@ -246,12 +388,12 @@ __device__ __noinline__ void jacobi_f32(float* A, float* Q, int n2, int max_swee
       const float v = A[i * LD + j];
       if (i == j) dia = fmaf(v, v, dia); else off = fmaf(v, v, off);
     }
-    off = block_reduce_f(off, reinterpret_cast<float*>(red), false);
-    dia = block_reduce_f(dia, reinterpret_cast<float*>(red), false);
+    off = block_sum_f<kThreads>(off, reinterpret_cast<float*>(red));
+    dia = block_sum_f<kThreads>(dia, reinterpret_cast<float*>(red));
     // off-diagonal mass below (1e-3)^2 of the diagonal: each float64 Newton step that follows
     // contracts the residual by about this factor (the next call refines the basis further)
     if (!(off > 1e-6 * dia)) break;
-    if (n2 == 64 && blockDim.x == kThreads) {
+    if constexpr (RPMAX == 64) if (n2 == 64) {
       // 32 pairs: every warp computes all 32 rotations itself (lane k: pair k) and takes the
       // ones it needs by shuffles, so a step needs a single barrier; a thread rotates the two
       // 2 x 2 blocks (pair w + 16u, pair lane) of A and the four (row w + 16u v, pair lane)
@@ -341,16 +483,11 @@ __device__ __noinline__ void jacobi_f32(float* A, float* Q, int n2, int max_swee
       // (rows {p1, q1}, columns {p2, q2}) is touched by exactly one row and one column rotation.
       // Each thread takes up to four blocks, loads all of them, then rotates and stores.
       {
-        constexpr int MB = (RPMAX / 2) * (RPMAX / 2) / kThreads;
+        constexpr int MB = ((RPMAX / 2) * (RPMAX / 2) + kThreads - 1) / kThreads;
         float v[MB][4];
         int pos[MB][4];
         float rc[MB][4];
         bool act[MB];
-        // with 32 pairs a thread's column pair k2 is its lane for every u: load it once
-        const bool lanepair = np == 32;
-        const int kl = threadIdx.x & 31;
-        const float cl = cs[kl], sl = sn[kl];
-        const int pl = pp[kl], ql = qq[kl];
 #pragma unroll
         for (int u = 0; u < MB; ++u) {
           const int e = threadIdx.x + u * kThreads;
@@ -358,10 +495,10 @@ __device__ __noinline__ void jacobi_f32(float* A, float* Q, int n2, int max_swee
           if (!act[u]) continue;
           const int k1 = pow2 ? (e >> lg) : e / np, k2 = pow2 ? (e & (np - 1)) : e % np;
           rc[u][0] = cs[k1]; rc[u][1] = sn[k1];
-          rc[u][2] = lanepair ? cl : cs[k2];
-          rc[u][3] = lanepair ? sl : sn[k2];
+          rc[u][2] = cs[k2];
+          rc[u][3] = sn[k2];
           act[u] = !(rc[u][1] == 0.f && rc[u][3] == 0.f);
-          const int p1 = pp[k1], q1 = qq[k1], p2 = lanepair ? pl : pp[k2], q2 = lanepair ? ql : qq[k2];
+          const int p1 = pp[k1], q1 = qq[k1], p2 = pp[k2], q2 = qq[k2];
           pos[u][0] = p1 * LD + p2; pos[u][1] = p1 * LD + q2; pos[u][2] = q1 * LD + p2; pos[u][3] = q1 * LD + q2;
 #pragma unroll
           for (int w = 0; w < 4; ++w) v[u][w] = A[pos[u][w]];
@@ -380,25 +517,21 @@ __device__ __noinline__ void jacobi_f32(float* A, float* Q, int n2, int max_swee
       }
       // Q <- Q J, up to eight (row, pair) items per thread, loads first
       {
-        constexpr int MQ = (RPMAX / 2) * RPMAX / kThreads;
+        constexpr int MQ = (RPMAX / 2 * RPMAX + kThreads - 1) / kThreads;
         float x2[MQ][2], cq[MQ][2];
         int qp[MQ][2];
         bool act[MQ];
-        const bool lanepair = np == 32;
-        const int kl = threadIdx.x & 31;
-        const float cl = cs[kl], sl = sn[kl];
-        const int pl = pp[kl], ql = qq[kl];
 #pragma unroll
         for (int u = 0; u < MQ; ++u) {
           const int e = threadIdx.x + u * kThreads;
           act[u] = e < np * n2;
           if (!act[u]) continue;
           const int k = pow2 ? (e & (np - 1)) : e % np, j = pow2 ? (e >> lg) : e / np;
-          cq[u][0] = lanepair ? cl : cs[k];
-          cq[u][1] = lanepair ? sl : sn[k];
+          cq[u][0] = cs[k];
+          cq[u][1] = sn[k];
           act[u] = cq[u][1] != 0.f;
-          qp[u][0] = j * LD + (lanepair ? pl : pp[k]);
-          qp[u][1] = j * LD + (lanepair ? ql : qq[k]);
+          qp[u][0] = j * LD + (pp[k]);
+          qp[u][1] = j * LD + (qq[k]);
           x2[u][0] = Q[qp[u][0]]; x2[u][1] = Q[qp[u][1]];
         }
 #pragma unroll
@@ -414,32 +547,32 @@ __device__ __noinline__ void jacobi_f32(float* A, float* Q, int n2, int max_swee
   }
 }
 
-// A = (B Q)^T G (B Q) kn = kn Q^T K Q for the float32 copies Bf, Gf (three products; K itself is
-// never formed).  The padding row and column r of an odd-sized Jacobi problem (n2 = r + 1) are zero.
-__device__ __noinline__ void gram_in_basis(const float* Bf, const float* Gf, const float* Q, float* A, float* F1,
-                                           float* F2, int r, int n2, float kn) {
-  mmf<false, false>(Bf, Q, F1, r);   // B Q
-  mmf<false, false>(Gf, F1, F2, r);  // G B Q
-  mmf<true, false>(F1, F2, A, r);    // (B Q)^T G B Q
-  for (int e = threadIdx.x; e < n2 * n2; e += blockDim.x) {
-    const int i = e / n2, j = e % n2;
-    A[i * LD + j] = (i < r && j < r) ? A[i * LD + j] * kn : 0.f;
-  }
-  __syncthreads();
+// A = (B Q)^T G (B Q) f = f Q^T K Q for the float32 copies Bf, Gf (three products; K itself is never formed).
+template <typename DM>
+__device__ __forceinline__ void gram_in_basis(const float* Bf, const float* Gf, const float* Q, float* A, float* F1, float* F2,
+                                              int r, float f) {
+  mmf<DM, false>(Bf, Q, F1, r, Epi::kStore);   // B Q
+  mmf<DM, false>(Gf, F1, F2, r, Epi::kStore);  // G B Q
+  EpiArgs e;
+  e.f = f;
+  mmf<DM, true>(F1, F2, A, r, Epi::kScale, e);  // (B Q)^T G B Q
 }
 
-// One first-order eigenbasis refinement round for a nearly diagonal A = Q^T K Q / s (float32):
+// One first-order eigenbasis refinement round for a nearly diagonal f A = Q^T K Q / s (float32):
 // Q <- Q (I + E), E_pq = A_pq / (A_qq - A_pp) for p != q (the small-angle Jacobi rotation of
 // every pair at once), then one Newton-Schulz re-orthonormalisation, and the second-order
-// eigenvalue estimates lam_p = A_pp - sum_q A_pq E_pq (A itself is not recomputed).  Pairs with
+// eigenvalue estimates lam_p = f (A_pp - sum_q A_pq E_pq) (A itself is not recomputed; f is a power of two).  Pairs with
 // (relative) gaps below 1e-5 are left alone, since any basis of a cluster serves the Newton
 // preconditioner.  Returns max |E|; above 0.25 (A not close enough to diagonal for the
-// first-order step) nothing is changed.
-__device__ __noinline__ float refine_round(float* Q, const float* A, float* F1, float* F2, float* lam, int r,
-                                           double* red) {
+// first-order step) nothing is changed, else Q holds the refined basis and QT its transpose.
+template <typename DM>
+__device__ __noinline__ float refine_round(float* Q, float* QT, const float* A, float f, float* F1, float* F2,
+                                           float* lam, int r, unsigned* slot) {
+  constexpr int LD = DM::LD, RP = DM::RP;
   float big = 0.f;
-  for (int e = threadIdx.x; e < r * r; e += blockDim.x) {
-    const int p = e / r, q = e % r;
+  for (int e = threadIdx.x; e < r * RP; e += DM::NT) {
+    const int p = e / RP, q = e % RP;
+    if (q >= r) continue;
     float v = 0.f;
     if (p != q) {
       const float gap = A[q * LD + q] - A[p * LD + p];
@@ -449,53 +582,26 @@ __device__ __noinline__ float refine_round(float* Q, const float* A, float* F1, 
     F1[p * LD + q] = v;
     big = fmaxf(big, fabsf(v));
   }
-  big = block_reduce_f(big, reinterpret_cast<float*>(red), true);
+  big = block_max_f(big, slot);
   if (!(big <= 0.25f)) return big;
   // lam_p = A_pp - sum_q A_pq E_pq: one warp per row
-  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int p = threadIdx.x >> 5; p < r; p += nw) {
+  const int lane = threadIdx.x & 31;
+  for (int p = threadIdx.x >> 5; p < r; p += DM::NT / 32) {
     float acc = 0.f;
     for (int q = lane; q < r; q += 32) acc = fmaf(A[p * LD + q], F1[p * LD + q], acc);
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) lam[p] = A[p * LD + p] - acc;
+    if (lane == 0) lam[p] = (A[p * LD + p] - acc) * f;
   }
-  mmf<false, false>(Q, F1, F2, r);                  // Q E (ends with a barrier)
-  for (int e = threadIdx.x; e < r * r; e += blockDim.x) {
-    const int i = e / r, j = e % r;
-    Q[i * LD + j] += F2[i * LD + j];
-  }
-  __syncthreads();
-  mmf<true, false>(Q, Q, F1, r);                    // Q^T Q
-  for (int e = threadIdx.x; e < r * r; e += blockDim.x) {
-    const int i = e / r, j = e % r;
-    F1[i * LD + j] = 0.5f * ((i == j ? 3.f : 0.f) - F1[i * LD + j]);
-  }
-  __syncthreads();
-  mmf<false, false>(Q, F1, F2, r);                  // Q (3I - Q^T Q) / 2
-  for (int e = threadIdx.x; e < r * r; e += blockDim.x) Q[(e / r) * LD + e % r] = F2[(e / r) * LD + e % r];
-  __syncthreads();
+  EpiArgs e;
+  e.x = Q;
+  mmf<DM, false>(Q, F1, F2, r, Epi::kAdd, e);       // Q (I + E)
+  mmf<DM, true>(F2, F2, F1, r, Epi::kOrtho);        // (3 I - Q^T Q) / 2
+  e.ct = QT;
+  mmf<DM, false>(F2, F1, Q, r, Epi::kBoth, e);      // Q (3 I - Q^T Q) / 2
   return big;
 }
 
-struct RxrSmem {
-  double G[RPMAX * LDD];   // Gram of the thin factor (float64 sum of the partials); later B_bar
-  double T[RPMAX * LDD];   // T_hat = B Z_hat (Newton iterate); scratch vectors of the rank test
-  double W[RPMAX * LDD];   // B (until T_hat exists), then G T_hat
-  float Gf[RPMAX * LD];    // G 2^-eg (float32; the power of two keeps K = B G B finite)
-  float Bf[RPMAX * LD];    // B 2^-eb
-  float QT[RPMAX * LD];    // Q^T
-  float Af[RPMAX * LD];    // Q^T K Q / s (K = B G B), the Jacobi matrix, then the Newton correction in that basis
-  float Qf[RPMAX * LD];    // approximate eigenbasis of K
-  float F1[RPMAX * LD];    // scratch
-  float F2[RPMAX * LD];    // scratch
-  float lam[RPMAX], sq[RPMAX], isq[RPMAX];
-  double red[32];
-  float cs[RPMAX / 2], sn[RPMAX / 2];
-  int pp[RPMAX / 2], qq[RPMAX / 2];
-  double scale, inv_s, rs;  // s = trace(B G B) / r, 1 / s, 1 / sqrt(s)  (written by thread 0)
-  float kn;                 // r / trace of the scaled float32 K
-  int ok;
-};
+static_assert(sizeof(RxrSmem<64>) <= 232448, "shared memory per CTA");
 
 // Epilogues of mm_dist: the product itself, or I - product / s rounded to float32.
 struct PlainEpi {
@@ -527,6 +633,7 @@ __device__ __forceinline__ int exponent_of(long long bits) { return bits ? (int)
 // and the Newton corrections, which only steer the iteration.  The mixed path also forms the
 // starting T_hat = B Z0 and T_C in float32 (its U, V and C are float32).  Outputs are written by
 // rows, each CTA of the cluster its own slice.
+template <int RP>
 __device__ __forceinline__ void rxr_body(const VGrid& vg__, const double* __restrict__ Gg, int rp, int r,
                                          double* __restrict__ Bg, double* __restrict__ Tout,
                                          double* __restrict__ TCout, const float* __restrict__ Qin,
@@ -534,47 +641,58 @@ __device__ __forceinline__ void rxr_body(const VGrid& vg__, const double* __rest
   pdl_enter();
   SFR_VGRID(vg__);
   if (stopped(st)) return;
+  using DM = Dim<RP>;
+  constexpr int NT = DM::NT, LD = DM::LD, LDD = DM::LDD;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  RxrSmem& S = *reinterpret_cast<RxrSmem*>(smem_raw);
-  float* redf = reinterpret_cast<float*>(S.red);
+  RxrSmem<RP>& S = *reinterpret_cast<RxrSmem<RP>*>(smem_raw);
   cg::cluster_group cl = cg::this_cluster();
   const int tid = threadIdx.x;
   const int cs = (int)cl.num_blocks(), crank = (int)cl.block_rank();
   const bool writer = crank == 0;
   const int rpc = (r + cs - 1) / cs, row0 = min(r, crank * rpc), row1 = min(r, row0 + rpc);  // own rows
   const int n2 = (r + 1) & ~1;  // Jacobi works on an even size (row / column r zero when r is odd)
+  float* Q = S.Q;
   // 1. G and B in float64 (B in W until T_hat exists), their power-of-two-scaled float32 copies,
   //    and the warm-start eigenbasis (Qin)
-  constexpr int PER = RPMAX * RPMAX / kThreads;
-  double gv[PER], bv[PER];
-  long long gmax = 0, bmax = 0;
+  constexpr int PER = RP * RP / NT;
+  {
+    double gv[PER], bv[PER];
+    float qv[PER];
+    long long gmax = 0, bmax = 0;
 #pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const int e = tid + q * kThreads, i = e / RPMAX, j = e % RPMAX;
-    const bool in = i < r && j < r;
-    gv[q] = in ? Gg[i * rp + j] : 0.0;
-    bv[q] = in ? Bg[i * rp + j] : 0.0;
-    gmax = max(gmax, abs_bits(gv[q]));
-    bmax = max(bmax, abs_bits(bv[q]));
-  }
-  load_sq(Qin, rp, r, n2, S.Qf, 1.f);
-  gmax = block_max_ll(gmax, S.red);
-  bmax = block_max_ll(bmax, S.red);
-  if (gmax >= kInfBits || bmax >= kInfBits || bmax == 0) { fail(st, SFR_E_NAN); return; }
-  const int eg = exponent_of(gmax), eb = exponent_of(bmax);
+    for (int q = 0; q < PER; ++q) {
+      const int e = tid + q * NT, i = e / RP, j = e % RP;
+      const bool in = i < r && j < r;
+      gv[q] = in ? Gg[i * rp + j] : 0.0;
+      bv[q] = in ? Bg[i * rp + j] : 0.0;
+      qv[q] = in ? Qin[i * rp + j] : 0.f;
+    }
+    if (tid < 16) S.mx[tid] = 0;
 #pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const int e = tid + q * kThreads, i = e / RPMAX, j = e % RPMAX;
-    S.G[i * LDD + j] = gv[q];
-    S.W[i * LDD + j] = bv[q];
-    S.Gf[i * LD + j] = f64_to_f32_shift(gv[q], eg);
-    S.Bf[i * LD + j] = f64_to_f32_shift(bv[q], eb);
+    for (int q = 0; q < PER; ++q) {
+      gmax = max(gmax, abs_bits(gv[q]));
+      bmax = max(bmax, abs_bits(bv[q]));
+    }
+    block_max2_ll<NT>(gmax, bmax, S.red);
+    if (gmax >= kInfBits || bmax >= kInfBits || bmax == 0) { fail(st, SFR_E_NAN); return; }
+    const int eg_ = exponent_of(gmax), eb_ = exponent_of(bmax);
+    if (tid == 0) S.pp[0] = eg_, S.qq[0] = eb_;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      const int e = tid + q * NT, i = e / RP, j = e % RP;
+      S.G[i * LDD + j] = gv[q];
+      S.W[i * LDD + j] = bv[q];
+      S.Gf[i * LD + j] = f64_to_f32_shift(gv[q], eg_);
+      S.Bf[i * LD + j] = f64_to_f32_shift(bv[q], eb_);
+      Q[i * LD + j] = qv[q];
+    }
   }
   __syncthreads();
-  // 2. A = Q^T K Q in the previous call's basis Q (float32, from the scaled copies:
-  //    K 2^-(eg + 2 eb)); s = trace(K) / r = trace(A) / r; A <- A / s
-  gram_in_basis(S.Bf, S.Gf, S.Qf, S.Af, S.F1, S.F2, r, n2, 1.f);
-  const float trf = block_reduce_f(tid < r ? S.Af[tid * LD + tid] : 0.f, redf, false);
+  const int eg = S.pp[0], eb = S.qq[0];
+  // 2. A = Q^T K Q in the warm-start basis Q (float32, from the scaled copies: K 2^-(eg + 2 eb));
+  //    s = trace(K) / r = trace(A) / r; A's scale over s is the power of two kn
+  gram_in_basis<DM>(S.Bf, S.Gf, Q, S.Af, S.F1, S.F2, r, 1.f);
+  const float trf = warp_sum64(S.Af, LD + 1, r);
   if (tid == 0) {
     // s = 2^(2k), the even power of two nearest below trace(B G B) / r (within a factor 4 of
     // it), so that 1 / s and 1 / sqrt(s) are exact and need no float64 division or square root;
@@ -593,142 +711,139 @@ __device__ __forceinline__ void rxr_body(const VGrid& vg__, const double* __rest
   __syncthreads();
   if (!S.ok) { fail(st, SFR_E_NAN); return; }
   const float kn = S.kn;
-  for (int e = tid; e < r * r; e += blockDim.x) S.Af[(e / r) * LD + e % r] *= kn;
-  __syncthreads();
   // 3. eigenbasis: refine the previous basis to first order (cheap) while its rotation is small;
   //    a round whose rotation is at most 1e-3 leaves the basis accurate to ~1e-6 and is the last,
   //    a larger one is followed by a fresh A; float32 Jacobi sweeps only when that does not converge
   bool accepted = false;
+  float fa = kn;  // scale of A
+  int slot = 0;
   for (int round = 0; round < 3 && !accepted; ++round) {
-    const float big = refine_round(S.Qf, S.Af, S.F1, S.F2, S.lam, n2, S.red);
+    const float big = refine_round<DM>(Q, S.QT, S.Af, fa, S.F1, S.F2, S.lam, r, S.mx + slot++);
     if (!(big <= 0.25f)) break;                      // A unchanged, Q unchanged
     accepted = big <= 1e-3f;
-    if (!accepted) gram_in_basis(S.Bf, S.Gf, S.Qf, S.Af, S.F1, S.F2, r, n2, kn);
+    if (!accepted) {
+      gram_in_basis<DM>(S.Bf, S.Gf, Q, S.Af, S.F1, S.F2, r, kn);
+      fa = 1.f;
+    }
   }
   const bool rotated = !accepted;
   if (rotated) {
-    jacobi_f32(S.Af, S.Qf, n2, 10, S.red, S.cs, S.sn, S.pp, S.qq);
-    // re-orthonormalise the float basis: Q <- Q (3I - Q^T Q) / 2
-    mmf<true, false>(S.Qf, S.Qf, S.F1, r);
-    for (int e = tid; e < r * r; e += blockDim.x) {
-      const int i = e / r, j = e % r;
-      S.F1[i * LD + j] = 0.5f * ((i == j ? 3.f : 0.f) - S.F1[i * LD + j]);
+    // A in K / s's scale, padded to an even size
+    for (int e = tid; e < n2 * RP; e += NT) {
+      const int i = e / RP, j = e % RP;
+      if (j >= n2) continue;
+      const bool in = i < r && j < r;
+      S.Af[i * LD + j] = in ? S.Af[i * LD + j] * fa : 0.f;
+      if (!in) Q[i * LD + j] = i == j ? 1.f : 0.f;
     }
     __syncthreads();
-    mmf<false, false>(S.Qf, S.F1, S.F2, r);
-    for (int e = tid; e < r * r; e += blockDim.x) S.Qf[(e / r) * LD + e % r] = S.F2[(e / r) * LD + e % r];
-    __syncthreads();
+    jacobi_f32<DM>(S.Af, Q, n2, 10, S.red, S.cs, S.sn, S.pp, S.qq);
+    // re-orthonormalise the float basis: Q <- Q (3I - Q^T Q) / 2
+    mmf<DM, true>(Q, Q, S.F1, r, Epi::kOrtho);
+    EpiArgs ec;
+    ec.ct = S.QT;
+    mmf<DM, false>(Q, S.F1, S.F2, r, Epi::kBoth, ec);
+    for (int e = tid; e < r * RP; e += NT)
+      if (e / RP < r && e % RP < r) Q[(e / RP) * LD + e % RP] = S.F2[(e / RP) * LD + e % RP];
     // 4. eigenvalue estimates after Jacobi: the diagonal of A (Rayleigh quotients of the basis)
-    for (int p = tid; p < r; p += blockDim.x) S.lam[p] = S.Af[p * LD + p];
+    for (int p = tid; p < r; p += NT) S.lam[p] = S.Af[p * LD + p];
+    __syncthreads();
   }
   // (after a refinement round lam holds its second-order estimates); those far below the largest
   // are recomputed in float64 for the rank test (Eq. 9 needs rank r)
-  __syncthreads();
-  float hi = 0.f;
-  for (int p = tid; p < r; p += blockDim.x) hi = fmaxf(hi, S.lam[p]);
-  hi = block_reduce_f(hi, redf, true);
-  float anysmall = 0.f;
-  for (int p = tid; p < r; p += blockDim.x)
-    if (S.lam[p] < 1e-6f * hi) anysmall = 1.f;
-  anysmall = block_reduce_f(anysmall, redf, true);
-  if (anysmall > 0.f && rotated) {
-    // Jacobi stopped at a 1e-3 off-diagonal, so a basis vector of a tiny eigenvalue still mixes
-    // ~1e-3 of the large ones and its Rayleigh quotient sits near 1e-6 hi: two first-order rounds
-    // (near-degenerate pairs are skipped) bring the mixing down to float32 rounding first.
-    for (int round = 0; round < 2; ++round) {
-      gram_in_basis(S.Bf, S.Gf, S.Qf, S.Af, S.F1, S.F2, r, n2, kn);
-      if (!(refine_round(S.Qf, S.Af, S.F1, S.F2, S.lam, n2, S.red) <= 0.25f)) {
-        for (int p = tid; p < r; p += blockDim.x) S.lam[p] = S.Af[p * LD + p];
-        break;
+  LamStats ls = lam_stats(S.lam, r);
+  if (ls.small) {
+    if (rotated) {
+      // Jacobi stopped at a 1e-3 off-diagonal, so a basis vector of a tiny eigenvalue still mixes
+      // ~1e-3 of the large ones and its Rayleigh quotient sits near 1e-6 hi: two first-order rounds
+      // (near-degenerate pairs are skipped) bring the mixing down to float32 rounding first.
+      __syncthreads();
+      for (int round = 0; round < 2; ++round) {
+        gram_in_basis<DM>(S.Bf, S.Gf, Q, S.Af, S.F1, S.F2, r, kn);
+        if (!(refine_round<DM>(Q, S.QT, S.Af, 1.f, S.F1, S.F2, S.lam, r, S.mx + slot++) <= 0.25f)) {
+          for (int p = tid; p < r; p += NT) S.lam[p] = S.Af[p * LD + p];
+          break;
+        }
       }
+      __syncthreads();
+      ls.hi = lam_stats(S.lam, r).hi;
     }
+    // A float32 eigenvector carries components of about 1e-7 along the large eigenvectors, which
+    // alone would add ~1e-14 hi to its Rayleigh quotient (the rank threshold): project them out in
+    // float64 first (q <- q - Q_L Q_L^T q over the columns of large eigenvalues), then take
+    // q^T K q / (s q^T q) = (B q)^T G (B q) / (s q^T q) with float64 matrix-vector products.
+    const float hi = ls.hi;
+    double* qs = S.T;            // the vector (T_hat is free until step 6)
+    double* cf = S.T + LDD;      // its coefficients on the large eigenvectors
+    double* bq = S.T + 2 * LDD;  // B q
     __syncthreads();
-    hi = 0.f;
-    for (int p = tid; p < r; p += blockDim.x) hi = fmaxf(hi, S.lam[p]);
-    hi = block_reduce_f(hi, redf, true);
-  }
-  // A float32 eigenvector carries components of about 1e-7 along the large eigenvectors, which
-  // alone would add ~1e-14 hi to its Rayleigh quotient (the rank threshold): project them out in
-  // float64 first (q <- q - Q_L Q_L^T q over the columns of large eigenvalues), then take
-  // q^T K q / (s q^T q) = (B q)^T G (B q) / (s q^T q) with float64 matrix-vector products.
-  double* qs = S.T;            // the vector (T_hat is free until step 6)
-  double* cf = S.T + LDD;      // its coefficients on the large eigenvectors
-  double* bq = S.T + 2 * LDD;  // B q
-  for (int p = 0; anysmall > 0.f && p < r; ++p) {
-    if (!(S.lam[p] < 1e-6f * hi)) continue;  // uniform: lam is in shared memory
-    if (tid < r) qs[tid] = (double)S.Qf[tid * LD + p];
-    __syncthreads();
-    if (tid < r) {
-      double c = 0.0;
-      if (!(S.lam[tid] < 1e-6f * hi))
-        for (int k = 0; k < r; ++k) c = fma((double)S.Qf[k * LD + tid], qs[k], c);
-      cf[tid] = c;
-    }
-    __syncthreads();
-    double qi = 0.0;
-    if (tid < r) {
-      qi = qs[tid];
-      for (int q2 = 0; q2 < r; ++q2) qi = fma(-cf[q2], (double)S.Qf[tid * LD + q2], qi);
-    }
-    __syncthreads();
-    if (tid < r) qs[tid] = qi;
-    __syncthreads();
-    if (tid < r) {
-      double v = 0.0;
-      for (int k = 0; k < r; ++k) v = fma(S.W[tid * LDD + k], qs[k], v);  // (B q)_tid
-      bq[tid] = v;
-    }
-    __syncthreads();
-    double num = 0.0, den = 0.0;
-    if (tid < r) {
-      double gq = 0.0;
-      for (int k = 0; k < r; ++k) gq = fma(S.G[tid * LDD + k], bq[k], gq);  // (G B q)_tid
-      num = bq[tid] * gq;
-      den = qi * qi;
-    }
-    if (tid >= 64) num = den = 0.0;  // r <= 64: the first two warps hold every term
-    if (tid < 64) {
-      for (int o = 16; o > 0; o >>= 1) {
-        num += __shfl_xor_sync(0xffffffffu, num, o);
-        den += __shfl_xor_sync(0xffffffffu, den, o);
+    for (int p = 0; p < r; ++p) {
+      if (!(S.lam[p] < 1e-6f * hi)) continue;  // uniform: lam is in shared memory
+      if (tid < r) qs[tid] = (double)Q[tid * LD + p];
+      if (tid < 4) S.red[tid] = 0.0;
+      __syncthreads();
+      if (tid < r) {
+        double c = 0.0;
+        if (!(S.lam[tid] < 1e-6f * hi))
+          for (int k = 0; k < r; ++k) c = fma((double)Q[k * LD + tid], qs[k], c);
+        cf[tid] = c;
       }
+      __syncthreads();
+      double qi = 0.0;
+      if (tid < r) {
+        qi = qs[tid];
+        for (int q2 = 0; q2 < r; ++q2) qi = fma(-cf[q2], (double)Q[tid * LD + q2], qi);
+      }
+      __syncthreads();
+      if (tid < r) qs[tid] = qi;
+      __syncthreads();
+      if (tid < r) {
+        double v = 0.0;
+        for (int k = 0; k < r; ++k) v = fma(S.W[tid * LDD + k], qs[k], v);  // (B q)_tid
+        bq[tid] = v;
+      }
+      __syncthreads();
+      double num = 0.0, den = 0.0;
+      if (tid < r) {
+        double gq = 0.0;
+        for (int k = 0; k < r; ++k) gq = fma(S.G[tid * LDD + k], bq[k], gq);  // (G B q)_tid
+        num = bq[tid] * gq;
+        den = qi * qi;
+      }
+      if (tid < 64) {  // r <= 64: the first two warps hold every term
+        for (int o = 16; o > 0; o >>= 1) {
+          num += __shfl_xor_sync(0xffffffffu, num, o);
+          den += __shfl_xor_sync(0xffffffffu, den, o);
+        }
+        if ((tid & 31) == 0) S.red[tid >> 4] = num, S.red[(tid >> 4) + 1] = den;
+      }
+      __syncthreads();
+      if (tid == 0) S.lam[p] = (float)((S.red[0] + S.red[2]) / (S.red[1] + S.red[3]) * S.inv_s);
+      __syncthreads();
     }
-    if (tid == 0) S.red[0] = num, S.red[1] = den;
-    __syncthreads();
-    if (tid == 32) S.red[2] = num, S.red[3] = den;
-    __syncthreads();
-    if (tid == 0) S.lam[p] = (float)((S.red[0] + S.red[2]) / (S.red[1] + S.red[3]) * S.inv_s);
-    __syncthreads();
+    const LamStats l2 = lam_stats(S.lam, r);
+    // (thresholds against the estimate of the largest taken before the recomputation)
+    ls.lo = fminf(hi, l2.lo);
+    bool bad = false;
+    for (int p = 0; p < r; ++p) bad |= !(S.lam[p] > 1e-14f * hi);
+    ls.bad = bad || !(hi > 0.f);
   }
-  float nlo = -hi, badf = 0.f;  // max of -lambda and of the rank-failure flag
-  for (int p = tid; p < r; p += blockDim.x) {
-    nlo = fmaxf(nlo, -S.lam[p]);
-    if (!(S.lam[p] > 1e-14f * hi)) badf = 1.f;
-  }
-  const float lo = -block_reduce_f(nlo, redf, true);
-  const bool bad = block_reduce_f(badf, redf, true) > 0.f || !(hi > 0.f);
   if (writer && tid == 0) {
-    if (v_side) st->lam_min_v = (double)lo * S.scale; else st->lam_min_u = (double)lo * S.scale;
+    if (v_side) st->lam_min_v = (double)ls.lo * S.scale; else st->lam_min_u = (double)ls.lo * S.scale;
   }
-  if (bad) { fail(st, SFR_E_RANK); return; }
-  for (int p = tid; p < r; p += blockDim.x) {
+  if (ls.bad) { fail(st, SFR_E_RANK); return; }
+  for (int p = tid; p < r; p += NT) {
     const float sq = sqrtf(S.lam[p]);
     S.sq[p] = sq;
     S.isq[p] = 1.f / sq;
   }
   float* QT = S.QT;
-  for (int e = tid; e < r * r; e += blockDim.x) QT[(e % r) * LD + e / r] = S.Qf[(e / r) * LD + e % r];
   __syncthreads();
   // 5. Z0 = Q diag(lambda^{-1/2}) Q^T (float32 start; Newton below brings it to float64 accuracy)
-  for (int e = tid; e < r * r; e += blockDim.x) {
-    const int i = e / r, j = e % r;
-    S.F2[i * LD + j] = S.Qf[i * LD + j] * S.isq[j];
-  }
-  __syncthreads();
-  mmf<false, false>(S.F2, QT, S.F1, r);
-  for (int e = tid; e < r * r; e += blockDim.x) {
-    const int i = e / r, j = e % r;
-    S.F2[i * LD + j] = 0.5f * (S.F1[i * LD + j] + S.F1[j * LD + i]);
+  mmf<DM, false>(Q, QT, S.F1, r, Epi::kStore, EpiArgs(), S.isq);
+  for (int e = tid; e < r * RP; e += NT) {
+    const int i = e / RP, j = e % RP;
+    if (i < r && j < r) S.F2[i * LD + j] = 0.5f * (S.F1[i * LD + j] + S.F1[j * LD + i]);
   }
   __syncthreads();
   // 6. T_hat = B Z0.  Float64 path: float64 products of B with the float32 values of Z0, rows
@@ -738,58 +853,56 @@ __device__ __forceinline__ void rxr_body(const VGrid& vg__, const double* __rest
   //    rounding of U and V.
   const PlainEpi plain;
   if (mixed) {
-    mmf<false, false>(S.Bf, S.F2, S.F1, r);  // B Z0 2^-eb
-    for (int e = tid; e < r * r; e += blockDim.x) {
-      const int i = e / r, j = e % r;
-      S.T[i * LDD + j] = f32_to_f64_shift(S.F1[i * LD + j], eb);
+    mmf<DM, false>(S.Bf, S.F2, S.F1, r, Epi::kStore);  // B Z0 2^-eb
+    for (int e = tid; e < r * RP; e += NT) {
+      const int i = e / RP, j = e % RP;
+      if (j < r) S.T[i * LDD + j] = f32_to_f64_shift(S.F1[i * LD + j], eb);
     }
     __syncthreads();
     if (cs > 1) cl.sync();  // every CTA is past its reads of W (still B) before W rows arrive
   } else {
-    mm_dist<false>(S.W, S.F2, S.T, r, plain);
+    mm_dist<DM, false>(S.W, S.F2, S.T, r, plain);
   }
   // 7. Newton steps on Z K Z = I: R = I - T_hat^T (G T_hat) / s in float64, correction in float32
   bool w_stale = false;  // W lags T_hat by G (B Delta)
   for (int it = 0; it < 6; ++it) {
     // W was last read by the previous product (T_hat0 = B Z0 or the residual), F1 by this CTA
     // alone before that product's closing barrier: neither needs a barrier before its broadcast
-    mm_dist<false, false>(S.G, S.T, S.W, r, plain);               // W = G T_hat
-    mm_dist<true, false>(S.T, S.W, S.F1, r, ResidEpi{S.inv_s});  // I - Z K Z, rounded to float32
+    mm_dist<DM, false, false>(S.G, S.T, S.W, r, plain);               // W = G T_hat
+    mm_dist<DM, true, false>(S.T, S.W, S.F1, r, ResidEpi{S.inv_s});  // I - Z K Z, rounded to float32
     w_stale = false;
     float rmax = 0.f;
-    for (int e = tid; e < r * r; e += blockDim.x) rmax = fmaxf(rmax, fabsf(S.F1[(e / r) * LD + e % r]));
-    const float rm = block_reduce_f(rmax, redf, true);
+    for (int e = tid; e < r * RP; e += NT) {  // R = Sym(I - Z K Z)
+      const int i = e / RP, j = e % RP;
+      if (j >= r) continue;
+      const float v = S.F1[i * LD + j];
+      rmax = fmaxf(rmax, fabsf(v));
+      S.F2[i * LD + j] = 0.5f * (v + S.F1[j * LD + i]);
+    }
+    const float rm = block_max_f(rmax, S.mx + slot++);
     if (!(rm == rm)) { fail(st, SFR_E_NAN); return; }
     if (rm < 4e-16f * r) break;
-    for (int e = tid; e < r * r; e += blockDim.x) {  // R = Sym(I - Z K Z)
-      const int i = e / r, j = e % r;
-      S.F2[i * LD + j] = 0.5f * (S.F1[i * LD + j] + S.F1[j * LD + i]);
-    }
-    __syncthreads();
-    mmf<false, false>(S.F2, S.Qf, S.F1, r);    // R Q
-    mmf<true, false>(S.Qf, S.F1, S.Af, r);     // Q^T R Q
-    for (int e = tid; e < r * r; e += blockDim.x) {
-      const int p = e / r, q = e % r;
-      S.Af[p * LD + q] = __fdividef(S.Af[p * LD + q], S.sq[p] + S.sq[q]);
-    }
-    __syncthreads();
-    mmf<false, false>(S.Af, QT, S.F2, r);      // Dt Q^T
-    mmf<false, false>(S.Qf, S.F2, S.F1, r);    // Q Dt Q^T
-    for (int e = tid; e < r * r; e += blockDim.x) {
-      const int i = e / r, j = e % r;
-      S.F2[i * LD + j] = 0.5f * (S.F1[i * LD + j] + S.F1[j * LD + i]);  // Delta (symmetric)
-    }
-    __syncthreads();
-    mmf<false, false>(S.Bf, S.F2, S.F1, r);    // B Delta 2^-eb
-    // The step just taken leaves a residual of about (eigenbasis error + float32 rounding of the
+    // The step below leaves a residual of about (eigenbasis error + float32 rounding of the
     // correction) x rm + O(rm^2): from rm < 3e-6 about 1e-11 (mixed path, whose Gram carries
     // float32 rounding), from rm < 1e-7 about 1e-14 (float64 path), so stop without forming it again
     // and update only this CTA's rows of T_hat (the rows it writes).
     const bool last = rm < (mixed ? 3e-6f : 1e-7f) || it == 5;
-    const int e0 = last ? row0 * r : 0, e1 = last ? row1 * r : r * r;
-    for (int e = e0 + tid; e < e1; e += blockDim.x) {
-      const int i = e / r, j = e % r;
-      S.T[i * LDD + j] += f32_to_f64_shift(S.F1[i * LD + j], eb);
+    EpiArgs el;
+    el.x = S.sq;
+    mmf<DM, false>(S.F2, Q, S.F1, r, Epi::kStore);            // R Q
+    mmf<DM, true>(Q, S.F1, S.Af, r, Epi::kLyapunov, el);      // Dt = Q^T R Q / (sqrt(lam_p) + sqrt(lam_q))
+    mmf<DM, false>(S.Af, QT, S.F2, r, Epi::kStore);           // Dt Q^T
+    mmf<DM, false>(Q, S.F2, S.F1, r, Epi::kStore);            // Q Dt Q^T
+    for (int e = tid; e < r * RP; e += NT) {
+      const int i = e / RP, j = e % RP;
+      if (j < r) S.F2[i * LD + j] = 0.5f * (S.F1[i * LD + j] + S.F1[j * LD + i]);  // Delta (symmetric)
+    }
+    __syncthreads();
+    mmf<DM, false>(S.Bf, S.F2, S.F1, r, Epi::kStore);         // B Delta 2^-eb
+    const int lo = last ? row0 : 0, hi = last ? row1 : r;
+    for (int e = lo * RP + tid; e < hi * RP; e += NT) {
+      const int i = e / RP, j = e % RP;
+      if (j < r) S.T[i * LDD + j] += f32_to_f64_shift(S.F1[i * LD + j], eb);
     }
     __syncthreads();
     w_stale = true;
@@ -797,13 +910,13 @@ __device__ __forceinline__ void rxr_body(const VGrid& vg__, const double* __rest
   }
   // 8. T = B (B G B)^{-1/2} = T_hat / sqrt(s): this CTA's rows, and its rows of the basis
   const double rs = S.rs;
-  for (int e = row0 * rp + tid; e < row1 * rp; e += blockDim.x) {
+  for (int e = row0 * rp + tid; e < row1 * rp; e += NT) {
     const int i = e / rp, j = e % rp;
     Tout[e] = j < r ? S.T[i * LDD + j] * rs : 0.0;
-    Qeig[e] = j < r ? S.Qf[i * LD + j] : (i == j ? 1.f : 0.f);
+    Qeig[e] = j < r ? Q[i * LD + j] : (i == j ? 1.f : 0.f);
   }
   if (writer)
-    for (int e = r * rp + tid; e < rp * rp; e += blockDim.x) {  // padding rows
+    for (int e = r * rp + tid; e < rp * rp; e += NT) {  // padding rows
       const int i = e / rp, j = e % rp;
       Tout[e] = 0.0;
       Qeig[e] = i == j ? 1.f : 0.f;
@@ -812,9 +925,10 @@ __device__ __forceinline__ void rxr_body(const VGrid& vg__, const double* __rest
   // 9. B_bar = Sym(G_W T_V) (Eq. 10 with W = X^T U_bar) = Sym(G T_hat) / sqrt(s), T_C = T_V B_bar.
   //    W lags T_hat by the last correction: W + G (B Delta), the latter in float32.  Every CTA forms
   //    its rows of B_bar and sends them to the others (nobody reads G after the last W product).
-  if (w_stale) mmf<false, false>(S.Gf, S.F1, S.F2, r);  // G B Delta 2^-(eg + eb)
-  for (int e = row0 * r + tid; e < row1 * r; e += blockDim.x) {
-    const int i = e / r, j = e % r;
+  if (w_stale) mmf<DM, false>(S.Gf, S.F1, S.F2, r, Epi::kStore);  // G B Delta 2^-(eg + eb)
+  for (int e = tid; e < (row1 - row0) * RP; e += NT) {
+    const int i = row0 + e / RP, j = e % RP;
+    if (j >= r) continue;
     double v = S.W[i * LDD + j] + S.W[j * LDD + i];
     if (w_stale) v += f32_to_f64_shift(S.F2[i * LD + j] + S.F2[j * LD + i], eg + eb);
     S.G[i * LDD + j] = 0.5 * rs * v;
@@ -822,7 +936,7 @@ __device__ __forceinline__ void rxr_body(const VGrid& vg__, const double* __rest
   __syncthreads();
   if (cs > 1) {
     const int npc = (r + 1) / 2, per = (row1 - row0) * npc;
-    for (int e = tid; e < (cs - 1) * per; e += blockDim.x) {
+    for (int e = tid; e < (cs - 1) * per; e += NT) {
       const int q = 1 + e / per, w = e % per;
       const int i = row0 + w / npc, j = 2 * (w % npc);
       double* Gq = cl.map_shared_rank(S.G, (crank + q) % cs);
@@ -833,17 +947,15 @@ __device__ __forceinline__ void rxr_body(const VGrid& vg__, const double* __rest
   // this CTA's rows: B_bar, and T_C = T_V B_bar = (T_hat rows) B_bar / sqrt(s).  T_C only forms
   // C = W T_C, which the mixed path stores in float32: there float32 products suffice.
   if (mixed) {
-    for (int e = tid; e < r * r; e += blockDim.x) {
-      const int i = e / r, j = e % r;
+    for (int e = tid; e < r * RP; e += NT) {
+      const int i = e / RP, j = e % RP;
+      if (j >= r) continue;
       S.Af[i * LD + j] = f64_to_f32_shift(S.G[i * LDD + j], 0);
-    }
-    for (int e = row0 * r + tid; e < row1 * r; e += blockDim.x) {
-      const int i = e / r, j = e % r;
-      S.F2[i * LD + j] = f64_to_f32_shift(S.T[i * LDD + j], 0);
+      if (i >= row0 && i < row1) S.F2[i * LD + j] = f64_to_f32_shift(S.T[i * LDD + j], 0);
     }
     __syncthreads();
   }
-  for (int e = row0 * rp + tid; e < row1 * rp; e += blockDim.x) {
+  for (int e = row0 * rp + tid; e < row1 * rp; e += NT) {
     const int i = e / rp, j = e % rp;
     double tc = 0.0;
     if (j < r && mixed) {
@@ -867,7 +979,7 @@ __device__ __forceinline__ void rxr_body(const VGrid& vg__, const double* __rest
     TCout[e] = j < r ? tc * rs : 0.0;
   }
   if (writer)
-    for (int e = r * rp + tid; e < rp * rp; e += blockDim.x) {
+    for (int e = r * rp + tid; e < rp * rp; e += NT) {
       Bg[e] = 0.0;
       TCout[e] = 0.0;
     }
@@ -876,37 +988,37 @@ __device__ __forceinline__ void rxr_body(const VGrid& vg__, const double* __rest
 
 }  // namespace
 
-// Cluster size for the r x r kernel: 16 CTAs (non-portable size) when the device accepts it
-// with this kernel's shared memory, else 8, else a single CTA.  The result does not depend on
-// it (every float64 product element is one thread's loop; the float32 work is redundant).
-static int rxr_cluster_size(size_t smem) {
-  static int cached = 0;
-  if (cached) return cached;
-  auto kern = body_kernel_of<&rxr_body, kThreads>();
-  int best = 1;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
-    cudaGetLastError();
-  if (set_smem_attr<body_kernel_of<&rxr_body, kThreads>()>(smem) != cudaSuccess) cudaGetLastError();
-  for (int cs : {16, 8}) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(cs);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = cs;
-    at.val.clusterDim.y = 1;
-    at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    int nclusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&nclusters, kern, &cfg) == cudaSuccess && nclusters > 0) {
-      best = cs;
-      break;
+// Cluster size of the r x r kernel: one CTA for r <= 16 (a whole float64 product takes it about a
+// microsecond, no more than the cluster barriers of a split one); above, 16 CTAs (non-portable
+// size) when the device accepts it with this kernel's shared memory, else 8, else a single CTA.  The
+// result does not depend on it (every float64 product element is one thread's loop; the float32 work is redundant).
+template <int RP>
+static int rxr_cluster_size() {
+  if (RP <= 16) return 1;
+  static const int best = [] {
+    constexpr size_t smem = sizeof(RxrSmem<RP>);
+    constexpr int NT = Dim<RP>::NT;
+    auto kern = body_kernel_of<&rxr_body<RP>, NT>();
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) cudaGetLastError();
+    if (set_smem_attr<body_kernel_of<&rxr_body<RP>, NT>()>(smem) != cudaSuccess) cudaGetLastError();
+    for (int cs : {16, 8}) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(cs);
+      cfg.blockDim = dim3(NT);
+      cfg.dynamicSmemBytes = smem;
+      cudaLaunchAttribute at;
+      at.id = cudaLaunchAttributeClusterDimension;
+      at.val.clusterDim.x = cs;
+      at.val.clusterDim.y = 1;
+      at.val.clusterDim.z = 1;
+      cfg.attrs = &at;
+      cfg.numAttrs = 1;
+      int nclusters = 0;
+      if (cudaOccupancyMaxActiveClusters(&nclusters, kern, &cfg) == cudaSuccess && nclusters > 0) return cs;
+      cudaGetLastError();
     }
-    cudaGetLastError();
-  }
-  cached = best;
+    return 1;
+  }();
   return best;
 }
 
@@ -915,15 +1027,25 @@ cudaError_t launch_rxr(const Shape& s, const Buffers& b, bool v_side, cudaStream
   const int count = v_side ? s.gw_blocks : s.gp_blocks;
   cudaError_t e = launch_reduce_parts(parts, count, s.rp * s.rp, b.Gsum, b.st, st);
   if (e != cudaSuccess) return e;
-  const size_t smem = sizeof(RxrSmem);
-  const int cs = rxr_cluster_size(smem);
   // warm start: the U side from its own basis of the previous iteration; the V side from the U
   // side's basis of this iteration (both K share B, and their eigenbases meet as the iteration
   // settles, so the V side's first-order refinement holds from the fourth iteration on)
-  return launch_k_cluster<&rxr_body, kThreads>(cs, kThreads, smem, st, (const double*)b.Gsum, s.rp, s.r, b.B,
-                                              v_side ? b.TV : b.TU, v_side ? b.TCm : (double*)nullptr,
-                                              (const float*)b.Qeig_u, v_side ? b.Qeig_v : b.Qeig_u,
-                                              v_side ? 1 : 0, fp64 ? 0 : 1, b.st);
+  auto go = [&](auto rpc) {
+    constexpr int RP = decltype(rpc)::value, NT = Dim<RP>::NT;
+    return launch_k_cluster<&rxr_body<RP>, NT>(rxr_cluster_size<RP>(), NT, sizeof(RxrSmem<RP>), st, (const double*)b.Gsum,
+                                              s.rp, s.r, b.B, v_side ? b.TV : b.TU, v_side ? b.TCm : (double*)nullptr,
+                                              (const float*)b.Qeig_u, v_side ? b.Qeig_v : b.Qeig_u, v_side ? 1 : 0,
+                                              fp64 ? 0 : 1, b.st);
+  };
+  // grouped launches use one kernel for every rank up to 32, so that a step has one projector launch
+  // per side whatever the ranks (which kernel runs a rank does not change its result)
+  if (g_recorder && s.rp <= 32) return go(std::integral_constant<int, 32>{});
+  switch (s.rp) {
+    case 8: return go(std::integral_constant<int, 8>{});
+    case 16: return go(std::integral_constant<int, 16>{});
+    case 32: return go(std::integral_constant<int, 32>{});
+    default: return go(std::integral_constant<int, 64>{});
+  }
 }
 
 }  // namespace sfr
