@@ -1573,6 +1573,51 @@ __global__ void import_kernel(const double* __restrict__ src, int64_t rows, int 
   dst[idx] = a < r ? (TC)src[i * r + a] : (TC)0;
 }
 
+// ---------------------------------------------------------------- grouped launches
+// The bodies of grouped launches (launch.cuh) take the padded rank at run time, so that all problems
+// of a step run in one launch per stage whatever their ranks: with one launch per rank (three of them in a
+// serving stream) each waited for the one before, and the CTAs of one rank alone did not fill the GPU.
+#define SFR_BY_RANK(rp, call)          \
+  do {                                 \
+    if ((rp) == 8) {                   \
+      constexpr int RP = 8;            \
+      call;                            \
+    } else if ((rp) == 16) {           \
+      constexpr int RP = 16;           \
+      call;                            \
+    } else {                           \
+      constexpr int RP = 32;           \
+      call;                            \
+    }                                  \
+  } while (0)
+
+__device__ __forceinline__ void thin_gram_any(const VGrid& vg, int rp, const float* parts, int nparts, int64_t part_stride,
+                                              float* out, int64_t rows, const float* addA, const double* H, double* gpart,
+                                              const DevState* st, const double* T2) {
+  SFR_BY_RANK(rp, (thin_gram_body<float, RP>(vg, parts, nparts, part_stride, out, rows, addA, H, gpart, st, 0, 0, T2,
+                                             nullptr, 0)));
+}
+__device__ __forceinline__ void row_transform_any(const VGrid& vg, int rp, const float* src, int64_t rows, const double* T,
+                                                  float* dst, const double* T2, float* dst2, const float* old,
+                                                  double* hpart, const DevState* st) {
+  SFR_BY_RANK(rp, (row_transform_body<float, RP>(vg, src, rows, T, dst, T2, dst2, old, hpart, st, nullptr, nullptr, nullptr,
+                                                 0, 0)));
+}
+template <typename TMs>
+__device__ __forceinline__ void sweep_mxp_any(const VGrid& vg, int rp, const TMs* M, int64_t m, int64_t n, int64_t ldm,
+                                              int64_t ldy, const float* Yin, float* Yout, float* D, const float* U,
+                                              const float* C, const float* V, float* Qpart, int cols_per_split,
+                                              double* resid_part, int r, const DevState* st) {
+  SFR_BY_RANK(rp, (sweep_mxp_body<TMs, RP>(vg, M, m, n, ldm, ldy, Yin, Yout, D, U, C, V, Qpart, cols_per_split, resid_part, r,
+                                           64, 2, st)));
+}
+template <typename TS>
+__device__ __forceinline__ void wpass_mxp_any(const VGrid& vg, int rp, const TS* src, int64_t lds, int64_t m, int64_t n,
+                                              int rows_per_chunk, const float* U, float* Wpart, const DevState* st) {
+  SFR_BY_RANK(rp, (wpass_mxp_body<TS, RP>(vg, src, lds, m, n, rows_per_chunk, U, Wpart, st)));
+}
+#undef SFR_BY_RANK
+
 // ---------------------------------------------------------------- dispatch helpers
 template <typename F>
 cudaError_t by_rank(int rp, F&& f) {
@@ -1711,6 +1756,10 @@ cudaError_t launch_gram_p(const Shape& s, const Buffers& b, bool fp64, bool sum_
           (const double*)nullptr, (const double*)nullptr, b.GPpart, b.st, 0, (int64_t)0, (const double*)nullptr,
           (__nv_bfloat16*)nullptr, (int64_t)0);
     });
+  if (g_recorder && s.rp <= 32)
+    return launch_k<&thin_gram_any, 256>(s.gp_blocks, 256, gram_smem<float, 32>(), st, s.rp,
+        static_cast<const float*>(b.Qpart), sum_parts ? s.nsplit : 0, s.m * s.rp, static_cast<float*>(b.P), s.m,
+        static_cast<const float*>(addA), H, b.GPpart, b.st, (const double*)nullptr);
   return by_rank(s.rp, [&](auto rpc) {
     constexpr int RP = decltype(rpc)::value;
     const size_t sm = gram_smem<float, RP>();
@@ -1737,6 +1786,10 @@ cudaError_t launch_apply_u(const Shape& s, const Buffers& b, bool fp64, bool fir
     return f64_transform(s, static_cast<const double*>(b.P), s.m, s.gp_blocks, b.TU, static_cast<double*>(b.U[u_new]),
                          nullptr, nullptr, first ? nullptr : static_cast<const double*>(b.U[u_old]),
                          first ? nullptr : b.Hpart, b.full ? nullptr : b.P, b.ex, nullptr, nullptr, b.st, st);
+  if (g_recorder && s.rp <= 32)
+    return launch_k<&row_transform_any, 256>(s.gp_blocks, 256, transform_smem<float, 32>(), st, s.rp,
+        static_cast<const float*>(b.P), s.m, b.TU, static_cast<float*>(b.U[u_new]), (const double*)nullptr, (float*)nullptr,
+        first ? nullptr : static_cast<const float*>(b.U[u_old]), first ? nullptr : b.Hpart, b.st);
   return by_rank(s.rp, [&](auto rpc) {
     constexpr int RP = decltype(rpc)::value;
     const size_t sm = transform_smem<float, RP>();
@@ -1773,6 +1826,9 @@ cudaError_t launch_wpass(const Shape& s, const Buffers& b, bool fp64, bool first
         };
         auto pipelined = [&](auto srcp, int64_t lds) {
           using TS = std::remove_const_t<std::remove_pointer_t<decltype(srcp)>>;
+          if (g_recorder)
+            return launch_k<&wpass_mxp_any<TS>, 256>(grid, 256, wxp_smem<TS, 32>(), st, RP, srcp, lds, s.m, s.n,
+                                                     s.rows_per_chunk, U, Wp, b.st);
           constexpr size_t sm = wxp_smem<TS, RP>();
           return launch_k<&wpass_mxp_body<TS, RP>, 256>(grid, 256, sm, st, srcp, lds, s.m, s.n, s.rows_per_chunk, U,
                                                          Wp, b.st);
@@ -1852,6 +1908,11 @@ cudaError_t launch_wfinal(const Shape& s, const Buffers& b, bool fp64, bool firs
   if (fp64)
     return f64_gram(s, static_cast<const double*>(b.Wpart), nparts, s.n * s.rp, static_cast<double*>(b.W), s.n, s.gw_blocks,
                     first ? nullptr : static_cast<const double*>(b.C), first ? nullptr : H, b.GWpart, b.st, st);
+  if (g_recorder && s.rp <= 32)
+    return launch_k<&thin_gram_any, 256>(s.gw_blocks, 256, gram_smem<float, 32>(), st, s.rp,
+        static_cast<const float*>(b.Wpart), nparts, s.n * s.rp, static_cast<float*>(b.W), s.n,
+        first ? nullptr : static_cast<const float*>(b.C), first ? nullptr : H, b.GWpart, b.st,
+        wp ? (const double*)b.TU : (const double*)nullptr);
   return by_rank(s.rp, [&](auto rpc) {
     constexpr int RP = decltype(rpc)::value;
     const size_t sm = gram_smem<float, RP>();
@@ -1878,6 +1939,10 @@ cudaError_t launch_apply_v(const Shape& s, const Buffers& b, bool fp64, cudaStre
                          static_cast<double*>(b.C), nullptr, nullptr, b.full ? nullptr : b.W, b.ex + tu + tv,
                          b.full ? nullptr : b.Wpart, b.ex + tu, b.st, st);
   }
+  if (g_recorder && s.rp <= 32)
+    return launch_k<&row_transform_any, 256>(s.gw_blocks, 256, transform_smem<float, 32>(), st, s.rp,
+        static_cast<const float*>(b.W), s.n, b.TV, static_cast<float*>(b.V), b.TCm, static_cast<float*>(b.C),
+        (const float*)nullptr, (double*)nullptr, b.st);
   return by_rank(s.rp, [&](auto rpc) {
     constexpr int RP = decltype(rpc)::value;
     const size_t sm = transform_smem<float, RP>();
@@ -1912,10 +1977,15 @@ static cudaError_t launch_sweep_mx(const Shape& s, const Buffers& b, int u_cur, 
         };
         if constexpr (!std::is_same<TMs, double>::value) {
           if (vec) {
+            if (g_recorder)
+              return launch_k<&sweep_mxp_any<TMs>, 256>(
+                  grid, 256, mxp_smem<TMs, 32>(64, 2), st, RP, M, s.m, s.n, s.ldm, b.ldy, static_cast<const float*>(b.Y[0]),
+                  static_cast<float*>(b.Y[1]), static_cast<float*>(b.D), static_cast<const float*>(b.U[u_cur]),
+                  static_cast<const float*>(b.C), static_cast<const float*>(b.V), static_cast<float*>(b.Qpart),
+                  s.cols_per_split, b.resid_part, s.r, b.st);
             // narrow matrices: as many columns as needed and up to four stages in half an SM's shared memory
-            // (grouped launches keep one shape, so that problems of different widths share a launch)
             int tw = 64, nst = 2;
-            if (!g_recorder && s.n <= 64) {
+            if (s.n <= 64) {
               tw = (int)(s.n + 7) / 8 * 8;
               while (nst < 4 && mxp_smem<TMs, RP>(tw, nst + 1) <= 110 * 1024) ++nst;
             }
