@@ -37,26 +37,27 @@ size_t solver_budget(const Solver& sv);
 
 namespace {
 
+// out[i][j] = M[perm[i]][j], i < rows, j < cols (a dense block of M~): one warp per row and 2048-byte
+// piece, 16 bytes per lane and step when every row starts on a 16-byte boundary (vec).
 template <typename T>
-__global__ void gather_cols_kernel(const T* __restrict__ M, int64_t ldm, const int64_t* __restrict__ perm, int64_t m,
-                                   int64_t l, T* __restrict__ out) {
+__global__ void __launch_bounds__(256) gather_kernel(const T* __restrict__ M, int64_t ldm, const int64_t* __restrict__ perm,
+                                                     int64_t rows, int64_t cols, T* __restrict__ out, int vec) {
   pdl_enter();
-  // out[i][j] = M[perm[i]][j], j < l   (left block of M~, m x l, dense)
-  int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= m * l) return;
-  int64_t i = idx / l, j = idx % l;
-  out[idx] = M[perm[i] * ldm + j];
-}
-
-template <typename T>
-__global__ void gather_rows_kernel(const T* __restrict__ M, int64_t ldm, const int64_t* __restrict__ perm, int64_t l,
-                                   int64_t n, T* __restrict__ out) {
-  pdl_enter();
-  // out[i][j] = M[perm[i]][j], i < l   (top block of M~, l x n, dense)
-  int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= l * n) return;
-  int64_t i = idx / n, j = idx % n;
-  out[idx] = M[perm[i] * ldm + j];
+  constexpr int64_t PIECE = 2048 / sizeof(T), PER16 = 16 / sizeof(T);
+  const int64_t pieces = (cols + PIECE - 1) / PIECE, total = rows * pieces;
+  const int lane = threadIdx.x & 31;
+  for (int64_t w = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); w < total; w += (int64_t)gridDim.x * 8) {
+    const int64_t i = w / pieces, j0 = (w % pieces) * PIECE, j1 = min(cols, j0 + PIECE);
+    const T* src = M + perm[i] * ldm;
+    T* dst = out + i * cols;
+    if (vec) {
+#pragma unroll 4
+      for (int64_t j = j0 + lane * PER16; j < j1; j += 32 * PER16)
+        *reinterpret_cast<uint4*>(dst + j) = *reinterpret_cast<const uint4*>(src + j);
+    } else {
+      for (int64_t j = j0 + lane; j < j1; j += 32) dst[j] = src[j];
+    }
+  }
 }
 
 // flag = 1 when some perm[i] lies outside [0, m): checked before any gather or scatter.
@@ -69,9 +70,30 @@ __global__ void check_perm_kernel(const int64_t* __restrict__ perm, int64_t m, i
 constexpr int CR = kMaxRank;
 constexpr int CLD = CR + 1;
 
-// One CTA: Core = B_L (A^T A)^{-1} B_L (U_L[:l]^T U_T) B_T with A = U_L[:l] B_L.
-__global__ void nys_core_kernel(const double* __restrict__ UL, const double* __restrict__ BL,
-                                const double* __restrict__ UT, const double* __restrict__ BT, int64_t l, int r,
+// Partial sums over the l rows: g1[p] = U_L^T U_L, g2[p] = U_L^T U_T (r x r each) over the rows of CTA p
+// (l / parts each).  A single CTA summing all rows took 1.8 ms at l = 2048, r = 20.
+__global__ void __launch_bounds__(256) nys_gram_kernel(const double* __restrict__ UL, const double* __restrict__ UT,
+                                                       int64_t l, int r, double* __restrict__ g1,
+                                                       double* __restrict__ g2) {
+  pdl_enter();
+  const int64_t i0 = blockIdx.x * l / gridDim.x, i1 = (blockIdx.x + 1) * l / gridDim.x;
+  for (int e = threadIdx.x; e < r * r; e += blockDim.x) {
+    const int a = e / r, b = e % r;
+    double s1 = 0.0, s2 = 0.0;
+#pragma unroll 4
+    for (int64_t i = i0; i < i1; ++i) {
+      const double u = UL[i * r + a];
+      s1 = fma(u, UL[i * r + b], s1);
+      s2 = fma(u, UT[i * r + b], s2);
+    }
+    g1[(int64_t)blockIdx.x * r * r + e] = s1;
+    g2[(int64_t)blockIdx.x * r * r + e] = s2;
+  }
+}
+
+// One CTA: Core = B_L (A^T A)^{-1} B_L (U_L[:l]^T U_T) B_T with A = U_L[:l] B_L, from the partial Gram sums.
+__global__ void nys_core_kernel(const double* __restrict__ g1p, const double* __restrict__ g2p, int parts,
+                                const double* __restrict__ BL, const double* __restrict__ BT, int r,
                                 double* __restrict__ core, int* __restrict__ bad) {
   pdl_enter();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -83,9 +105,10 @@ __global__ void nys_core_kernel(const double* __restrict__ UL, const double* __r
   for (int e = tid; e < r * r; e += blockDim.x) {
     const int a = e / r, b = e % r;
     double g1 = 0.0, g2 = 0.0;
-    for (int64_t i = 0; i < l; ++i) {
-      g1 = fma(UL[i * r + a], UL[i * r + b], g1);
-      g2 = fma(UL[i * r + a], UT[i * r + b], g2);
+#pragma unroll 8
+    for (int p = 0; p < parts; ++p) {
+      g1 += g1p[(int64_t)p * r * r + e];
+      g2 += g2p[(int64_t)p * r * r + e];
     }
     G1[a * CLD + b] = g1;
     G2[a * CLD + b] = g2;
@@ -190,35 +213,134 @@ __global__ void nys_rows_kernel(const double* __restrict__ UL, const double* __r
 }
 
 // S = M - Uo V_T^T (and optionally L), Algorithm 2's S = M~ - L in M's row order.
-template <typename TC, typename TMs, typename TSo>
+template <typename TMs, typename TSo>
 __global__ void __launch_bounds__(256) nys_residual_kernel(const TMs* __restrict__ M, int64_t m, int64_t n,
                                                            int64_t ldm, const double* __restrict__ Uo,
                                                            const double* __restrict__ VT, int r, TSo* __restrict__ S,
                                                            TSo* __restrict__ L, int64_t lds) {
   pdl_enter();
-  __shared__ TC us[8][CR];
-  __shared__ TC vs[32][CR + 1];
+  __shared__ double us[8][CR];
+  __shared__ double vs[32][CR + 1];
   const int64_t nbx = (n + 31) / 32;  // 1-D grid over (8-row, 32-column) blocks, columns fastest
   const int64_t i0 = ((int64_t)blockIdx.x / nbx) * 8, j0 = ((int64_t)blockIdx.x % nbx) * 32;
   const int tj = threadIdx.x & 31, ti = threadIdx.x >> 5;
   for (int e = threadIdx.x; e < 8 * r; e += blockDim.x) {
     int ii = e / r, a = e % r;
-    us[ii][a] = i0 + ii < m ? (TC)Uo[(i0 + ii) * r + a] : (TC)0;
+    us[ii][a] = i0 + ii < m ? (double)Uo[(i0 + ii) * r + a] : (double)0;
   }
   for (int e = threadIdx.x; e < 32 * r; e += blockDim.x) {
     int jj = e / r, a = e % r;
-    vs[jj][a] = j0 + jj < n ? (TC)VT[(j0 + jj) * r + a] : (TC)0;
+    vs[jj][a] = j0 + jj < n ? (double)VT[(j0 + jj) * r + a] : (double)0;
   }
   __syncthreads();
   const int64_t i = i0 + ti, j = j0 + tj;
   if (i >= m || j >= n) return;
-  TC lv = 0;
+  double lv = 0;
   for (int a = 0; a < r; ++a) lv += us[ti][a] * vs[tj][a];
-  TC mv;
-  if constexpr (std::is_same<TMs, __nv_bfloat16>::value) mv = (TC)__bfloat162float(M[i * ldm + j]);
-  else mv = (TC)M[i * ldm + j];
+  double mv;
+  if constexpr (std::is_same<TMs, __nv_bfloat16>::value) mv = (double)__bfloat162float(M[i * ldm + j]);
+  else mv = (double)M[i * ldm + j];
   if (S) S[i * lds + j] = (TSo)(mv - lv);
   if (L) L[i * lds + j] = (TSo)lv;
+}
+
+// The same in float32 arithmetic, 64 x 128 outputs per CTA: a thread forms 4 rows x 8 columns, the sum over the
+// ranks in order, operands in 16-byte reads from rank-chunk tiles; 16-byte accesses where M, S and L allow them (vec).
+// Bound by the 4 + 4 bytes per element it writes: 32768 x 32768, r = 20, L and S float32, 11.5 -> 3.9 ms
+// (one output per thread before, two shared-memory reads per multiply-add).
+constexpr int kNrRows = 64, kNrCols = 128, kNrK = 32;
+template <typename TMs, typename TSo>
+__global__ void __launch_bounds__(256) nys_residual_f32_kernel(const TMs* __restrict__ M, int64_t m, int64_t n, int64_t ldm,
+                                                               const double* __restrict__ Uo, const double* __restrict__ VT,
+                                                               int r, TSo* __restrict__ S, TSo* __restrict__ L,
+                                                               int64_t lds, int vec) {
+  pdl_enter();
+  __shared__ __align__(16) float us[kNrRows][kNrK + 4];
+  __shared__ __align__(16) float vs[kNrK][kNrCols + 4];
+  const int64_t nbx = (n + kNrCols - 1) / kNrCols;  // 1-D grid, columns fastest
+  const int64_t i0 = ((int64_t)blockIdx.x / nbx) * kNrRows, j0 = ((int64_t)blockIdx.x % nbx) * kNrCols;
+  const int t = threadIdx.x, tc = t & 15, tr = t >> 4;  // rows tr + 16 x, columns 4 tc + 64 h + c
+  float l[4][8];
+#pragma unroll
+  for (int x = 0; x < 4; ++x)
+#pragma unroll
+    for (int c = 0; c < 8; ++c) l[x][c] = 0.f;
+  for (int k0 = 0; k0 < r; k0 += kNrK) {
+    const int kn = min(kNrK, r - k0), k4 = (kn + 3) & ~3;  // (ranks kn .. k4 are zero)
+    __syncthreads();
+    for (int e = t; e < kNrRows * k4; e += 256) {
+      const int ii = e / k4, a = e % k4;
+      us[ii][a] = i0 + ii < m && a < kn ? (float)Uo[(i0 + ii) * r + k0 + a] : 0.f;
+    }
+    for (int e = t; e < kNrCols * k4; e += 256) {
+      const int jj = e / k4, a = e % k4;
+      vs[a][jj] = j0 + jj < n && a < kn ? (float)VT[(j0 + jj) * r + k0 + a] : 0.f;
+    }
+    __syncthreads();
+    for (int a4 = 0; a4 < k4; a4 += 4) {
+      float u[4][4];
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        const float4 w = *reinterpret_cast<const float4*>(&us[tr + 16 * x][a4]);
+        u[x][0] = w.x; u[x][1] = w.y; u[x][2] = w.z; u[x][3] = w.w;
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 v0 = *reinterpret_cast<const float4*>(&vs[a4 + q][4 * tc]);
+        const float4 v1 = *reinterpret_cast<const float4*>(&vs[a4 + q][64 + 4 * tc]);
+        const float v[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+          for (int c = 0; c < 8; ++c) l[x][c] = fmaf(u[x][q], v[c], l[x][c]);
+      }
+    }
+  }
+#pragma unroll
+  for (int x = 0; x < 4; ++x) {
+    const int64_t i = i0 + tr + 16 * x;
+    if (i >= m) continue;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int64_t j = j0 + 64 * h + 4 * tc;
+      const float* lv = l[x] + 4 * h;
+      float mv[4];
+      const bool vecm = S && (vec & 2) && j + 4 <= n;
+      if constexpr (sizeof(TMs) <= 4) {
+        if (vecm) {  // 4 elements of M at once
+          if constexpr (sizeof(TMs) == 4) {
+            const float4 w = __ldcs(reinterpret_cast<const float4*>(M + i * ldm + j));
+            mv[0] = w.x; mv[1] = w.y; mv[2] = w.z; mv[3] = w.w;
+          } else {
+            const uint2 w = __ldcs(reinterpret_cast<const uint2*>(M + i * ldm + j));
+            mv[0] = __uint_as_float(w.x << 16); mv[1] = __uint_as_float(w.x & 0xFFFF0000u);
+            mv[2] = __uint_as_float(w.y << 16); mv[3] = __uint_as_float(w.y & 0xFFFF0000u);
+          }
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        if (!vecm) mv[c] = 0.f;
+        if (S && !vecm && j + c < n) {
+          if constexpr (std::is_same<TMs, __nv_bfloat16>::value) mv[c] = __bfloat162float(M[i * ldm + j + c]);
+          else mv[c] = (float)M[i * ldm + j + c];
+        }
+      }
+      if ((vec & 1) && j + 4 <= n) {
+        if constexpr (sizeof(TSo) == 4) {
+          if (S) __stcs(reinterpret_cast<float4*>(S + i * lds + j), make_float4(mv[0] - lv[0], mv[1] - lv[1], mv[2] - lv[2], mv[3] - lv[3]));
+          if (L) __stcs(reinterpret_cast<float4*>(L + i * lds + j), make_float4(lv[0], lv[1], lv[2], lv[3]));
+          continue;
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (j + c < n) {
+          if (S) S[i * lds + j + c] = (TSo)(mv[c] - lv[c]);
+          if (L) L[i * lds + j + c] = (TSo)lv[c];
+        }
+    }
+  }
 }
 
 template <typename F>
@@ -356,8 +478,14 @@ sfr_status nys_solve_device(Solver& sv, const sfr_problem& p, const void* Mdev, 
   if (hflag) { *err = "FR-Nys: nys_perm has an entry outside [0, m)"; return SFR_E_INVAL; }
   e = by_mtype(p.m_dtype, Mdev, [&](auto M) {
     using T = std::remove_const_t<std::remove_pointer_t<decltype(M)>>;
-    launch_pdl(gather_cols_kernel<T>, cdiv(m * l, 256), 256, 0, st, M, p.ldm, perm_dev, m, l, static_cast<T*>(Mleft));
-    launch_pdl(gather_rows_kernel<T>, cdiv(l * n, 256), 256, 0, st, M, p.ldm, perm_dev, l, n, static_cast<T*>(Mtop));
+    auto gather = [&](int64_t rows, int64_t cols, void* out) {  // (the blocks start on 256-byte boundaries)
+      const bool vec = (uintptr_t)M % 16 == 0 && p.ldm * sizeof(T) % 16 == 0 && cols * sizeof(T) % 16 == 0;
+      const int64_t warps = rows * ((cols * (int64_t)sizeof(T) + 2047) / 2048);
+      launch_pdl(gather_kernel<T>, (unsigned)std::min<int64_t>(cdiv(warps, 8), 8192), 256, 0, st, M, p.ldm, perm_dev, rows, cols,
+                 static_cast<T*>(out), vec ? 1 : 0);
+    };
+    gather(m, l, Mleft);
+    gather(l, n, Mtop);
     return cudaGetLastError();
   });
   if (e != cudaSuccess) { *err = cudaGetErrorString(e); return SFR_E_CUDA; }
@@ -429,7 +557,12 @@ sfr_status nys_solve_device(Solver& sv, const sfr_problem& p, const void* Mdev, 
   const int core_smem = (int)(4 * sizeof(double) * CR * CLD);
   e = cudaFuncSetAttribute(nys_core_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, core_smem);
   if (e != cudaSuccess) { *err = cudaGetErrorString(e); return SFR_E_CUDA; }
-  launch_pdl(nys_core_kernel, 1, 256, core_smem, st, UL, BL, UT, BT, l, r, core, flag);
+  // Gram partials: in Uo, which is written after them, or (one part) where the SVD factors go
+  const int parts = (int)std::max<int64_t>(1, std::min<int64_t>((l + 63) / 64, m / (2 * r)));
+  double* g1 = parts > 1 ? Uo : Asvd;
+  double* g2 = parts > 1 ? Uo + (size_t)parts * r * r : Csvd;
+  launch_pdl(nys_gram_kernel, parts, 256, 0, st, UL, UT, l, r, g1, g2);
+  launch_pdl(nys_core_kernel, 1, 256, core_smem, st, g1, g2, parts, BL, BT, r, core, flag);
   launch_pdl(nys_rows_kernel, cdiv(m * r, 256), 256, 0, st, UL, core, perm_dev, m, r, Uo);
   cudaMemcpyAsync(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost, st);
   e = cudaStreamSynchronize(st);
@@ -461,16 +594,19 @@ sfr_status nys_solve_device(Solver& sv, const sfr_problem& p, const void* Mdev, 
   if (Sdev || Ldev) {
     const int64_t nblk = (int64_t)cdiv(n, 32) * cdiv(m, 8);
     if (nblk > 0x7fffffffLL) { *err = "FR-Nys output: m x n too large for one launch"; return SFR_E_INVAL; }
-    const unsigned grid = (unsigned)nblk;
     const bool fp64 = p.precision == SFR_PREC_FP64;
+    const unsigned grid = fp64 ? (unsigned)nblk : cdiv(n, kNrCols) * cdiv(m, kNrRows);
+    // bit 0: 16-byte stores to S and L, bit 1: loads of 4 elements of M (float32, bfloat16)
+    const int vec = (res->s_dtype == SFR_F32 && (uintptr_t)Sdev % 16 == 0 && (uintptr_t)Ldev % 16 == 0 && res->lds % 4 == 0 ? 1 : 0) |
+                    (p.m_dtype != SFR_F64 && (uintptr_t)Mdev % 16 == 0 && p.ldm % 4 == 0 ? 2 : 0);
     e = by_mtype(p.m_dtype, Mdev, [&](auto M) {
       using TMs = std::remove_const_t<std::remove_pointer_t<decltype(M)>>;
       if (res->s_dtype == SFR_F64) {
-        if (fp64) launch_pdl(nys_residual_kernel<double, TMs, double>, grid, 256, 0, st, M, m, n, p.ldm, Uo, VT, r, (double*)Sdev, (double*)Ldev, res->lds);
-        else launch_pdl(nys_residual_kernel<float, TMs, double>, grid, 256, 0, st, M, m, n, p.ldm, Uo, VT, r, (double*)Sdev, (double*)Ldev, res->lds);
+        if (fp64) launch_pdl(nys_residual_kernel<TMs, double>, grid, 256, 0, st, M, m, n, p.ldm, Uo, VT, r, (double*)Sdev, (double*)Ldev, res->lds);
+        else launch_pdl(nys_residual_f32_kernel<TMs, double>, grid, 256, 0, st, M, m, n, p.ldm, Uo, VT, r, (double*)Sdev, (double*)Ldev, res->lds, vec);
       } else {
-        if (fp64) launch_pdl(nys_residual_kernel<double, TMs, float>, grid, 256, 0, st, M, m, n, p.ldm, Uo, VT, r, (float*)Sdev, (float*)Ldev, res->lds);
-        else launch_pdl(nys_residual_kernel<float, TMs, float>, grid, 256, 0, st, M, m, n, p.ldm, Uo, VT, r, (float*)Sdev, (float*)Ldev, res->lds);
+        if (fp64) launch_pdl(nys_residual_kernel<TMs, float>, grid, 256, 0, st, M, m, n, p.ldm, Uo, VT, r, (float*)Sdev, (float*)Ldev, res->lds);
+        else launch_pdl(nys_residual_f32_kernel<TMs, float>, grid, 256, 0, st, M, m, n, p.ldm, Uo, VT, r, (float*)Sdev, (float*)Ldev, res->lds, vec);
       }
       return cudaGetLastError();
     });
