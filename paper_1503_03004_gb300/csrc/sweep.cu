@@ -35,7 +35,8 @@ __device__ __forceinline__ bool stopped(const DevState* st) { return *(volatile 
 // their fixed-order sum in the iteration end) do not depend on how many CTAs the sweep runs.  One
 // warp adds all 256 parts in float64: eight warps reducing their own with float64 shuffles took 40
 // float64 operations of the narrow pipe per row block, this takes 12.
-__device__ __forceinline__ void resid_store(const float* rs, double* __restrict__ resid_part, int64_t split, int64_t nrb,
+template <typename TR>
+__device__ __forceinline__ void resid_store(const TR* rs, double* __restrict__ resid_part, int64_t split, int64_t nrb,
                                             int64_t rb) {
   const int lane = threadIdx.x & 31;
   double v = (double)rs[lane];
@@ -97,6 +98,46 @@ __global__ void norm_m_kernel(const TMs* __restrict__ M, int64_t m, int64_t n, i
       a = fmaf(v, v, a);
     }
     acc += (double)a;
+  }
+  acc = block_sum(acc, red);
+  if (threadIdx.x == 0) part[blockIdx.x] = acc;
+}
+
+// The same for a matrix without gaps between its rows (ldm == n) and float32 or bfloat16 storage, as one array of
+// 16-byte pieces: a row of 40 floats kept 10 of a CTA's 256 threads busy (2^20 x 40: 1.75 ms, now 0.04).
+template <typename TMs>
+__global__ void __launch_bounds__(256) norm_flat_kernel(const TMs* __restrict__ M, int64_t count, double* part) {
+  pdl_enter();
+  __shared__ double red[32];
+  constexpr int64_t V = 16 / sizeof(TMs);
+  const int64_t nv = count / V, stride = (int64_t)gridDim.x * 256;
+  const uint4* v = reinterpret_cast<const uint4*>(M);
+  double acc = 0.0;
+  for (int64_t c = blockIdx.x * 256LL + threadIdx.x; c < nv; c += 4 * stride) {
+    uint4 w[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) w[u] = c + u * stride < nv ? __ldg(v + c + u * stride) : make_uint4(0, 0, 0, 0);
+    float a = 0.f;  // float32 over 16 or 32 squares, float64 from there on
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const uint32_t q[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if constexpr (sizeof(TMs) == 2) {
+          const float lo = __uint_as_float(q[k] << 16), hi = __uint_as_float(q[k] & 0xffff0000u);
+          a = fmaf(lo, lo, a);
+          a = fmaf(hi, hi, a);
+        } else {
+          const float x = __uint_as_float(q[k]);
+          a = fmaf(x, x, a);
+        }
+      }
+    }
+    acc += (double)a;
+  }
+  if (blockIdx.x == 0 && threadIdx.x < count - nv * V) {
+    const double x = (double)ld_as<float, TMs>(M + nv * V + threadIdx.x);
+    acc += x * x;
   }
   acc = block_sum(acc, red);
   if (threadIdx.x == 0) part[blockIdx.x] = acc;
@@ -1001,7 +1042,8 @@ __device__ __forceinline__ void sweep_mxp_body(const VGrid& vg__, const TMs* __r
   constexpr int LDU = RP + 4;  // padded U rows: the four rows a warp reads fall in different banks
   constexpr int QR = RP / 4;   // rank groups
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ float rs[256];
+  using TR = std::conditional_t<RP == 64, double, float>;  // a thread's residual sum (above rank 32: float64 throughout)
+  __shared__ TR rs[256];
   const int ldx = tw + 4;
   const int64_t jbeg = (int64_t)blockIdx.y * cols_per_split;
   const int64_t jend = min(n, jbeg + cols_per_split);
@@ -1042,13 +1084,13 @@ __device__ __forceinline__ void sweep_mxp_body(const VGrid& vg__, const TMs* __r
       float* cs = Cs + (ic & 1) * RP * BN;
       ++ic;
 #pragma unroll
-      for (int it = 0; it < (RP == 32 ? 8 : 4); ++it) {
+      for (int it = 0; it < (RP == 64 ? 16 : RP == 32 ? 8 : 4); ++it) {
         constexpr int JL = 32 / QR;  // columns a warp covers at a time
         const int l = t & 31, q = l % QR, sI = it & 3;
         const int jj = ((it >> 2) * 8 + (t >> 5)) * JL + l / QR, a = 4 * q + sI;
         if (jj >= BN) continue;
         const bool ok = j0 + jj < jend;
-        cp_async4(cs + a * BN + (((jj >> 2) ^ q) << 2) + (jj & 3), ok ? (const void*)(C + (j0 + jj) * RP + a) : (const void*)C,
+        cp_async4(cs + a * BN + (((jj >> 2) ^ (q & 7)) << 2) + (jj & 3), ok ? (const void*)(C + (j0 + jj) * RP + a) : (const void*)C,
                   ok ? 4 : 0);
       }
     }
@@ -1091,7 +1133,7 @@ __device__ __forceinline__ void sweep_mxp_body(const VGrid& vg__, const TMs* __r
     cp_async_commit();
   }
   float q[2][QA];
-  float resid = 0.f;
+  TR resid = 0;
   int64_t rb = blockIdx.x, rb_done = -1;
   int tile = 0, stage = 0, cu = 0;
   for (int64_t k = 0; k < total; ++k) {
@@ -1115,7 +1157,7 @@ __device__ __forceinline__ void sweep_mxp_body(const VGrid& vg__, const TMs* __r
       for (int x = 0; x < 2; ++x)
 #pragma unroll
         for (int c = 0; c < QA; ++c) q[x][c] = 0.f;
-      resid = 0.f;
+      resid = 0;
     }
     // phase A: L for rows 2 tr, 2 tr + 1 and the thread's two column groups
     const float* us = Us + cu * BM * LDU + 2 * tr * LDU;
@@ -1179,8 +1221,8 @@ __device__ __forceinline__ void sweep_mxp_body(const VGrid& vg__, const TMs* __r
           const float z = mv[c] - lv + y * inv_mu;
           const float y1 = fminf(1.f, fmaxf(-1.f, mu * z));
           const float d = y1 * dcoef - y * inv_mu;
-          const float dy = y1 - y;
-          resid += ok ? dy * dy : 0.f;
+          const TR dy = y1 - y;
+          resid += ok ? dy * dy : (TR)0;
           yn[c] = y1;
           dd[c] = d;
           xx[c] = ok ? lv + d : 0.f;  // X = L + Delta (0 outside the matrix)
@@ -1204,7 +1246,11 @@ __device__ __forceinline__ void sweep_mxp_body(const VGrid& vg__, const TMs* __r
 #pragma unroll
       for (int s4 = 0; s4 < 4; ++s4) {
         float v[QA];
-        if constexpr (QA == 4) {
+        if constexpr (QA == 8) {
+          const float4 w = *reinterpret_cast<const float4*>(vp + (jj + s4) * RP);
+          const float4 z = *reinterpret_cast<const float4*>(vp + (jj + s4) * RP + 4);
+          v[0] = w.x; v[1] = w.y; v[2] = w.z; v[3] = w.w; v[4] = z.x; v[5] = z.y; v[6] = z.z; v[7] = z.w;
+        } else if constexpr (QA == 4) {
           const float4 w = *reinterpret_cast<const float4*>(vp + (jj + s4) * RP);
           v[0] = w.x; v[1] = w.y; v[2] = w.z; v[3] = w.w;
         } else if constexpr (QA == 2) {
@@ -1333,7 +1379,10 @@ __device__ __forceinline__ void wpass_mx_body(const VGrid& vg__, const TS* __res
 }
 
 // The W pass above with cp.async staging: 32-row tiles of src and U in a 4-stage ring, three
-// tiles in flight while one is accumulated.  Needs the vector conditions (src rows 16-byte
+// tiles in flight while one is accumulated.  A thread forms 4 columns x 4 ranks from 16-byte reads (two per 16
+// multiply-adds; 2 columns x r/8 ranks took two per 2 to 8) over every RS-th row of a tile, RS = 64 / RP row
+// groups, whose sums are added through shared memory at the end: 2^20 x 40, r = 3 101 -> 66 us, 2048 x 2048, r = 40
+// 45 -> 27 us.  Needs the vector conditions (src rows 16-byte
 // aligned, n % 4 == 0) and float32 or bfloat16 src.
 constexpr int kWxStages = 4;
 template <typename TS, int RP>
@@ -1343,7 +1392,8 @@ __device__ __forceinline__ void wpass_mxp_body(const VGrid& vg__, const TS* __re
   pdl_enter();
   SFR_VGRID(vg__);
   if (stopped(st)) return;
-  constexpr int BR = 32, BN = kMxBN, QA = RP / 8, EPC = 16 / (int)sizeof(TS);
+  constexpr int BR = 32, BN = kMxBN, EPC = 16 / (int)sizeof(TS);
+  constexpr int RS = 64 / RP;                // row groups
   constexpr int XS = BR * BN, US = BR * RP;  // elements per stage
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TS* Xs = reinterpret_cast<TS*>(smem_raw);                                  // [stages][BR][BN]
@@ -1352,7 +1402,7 @@ __device__ __forceinline__ void wpass_mxp_body(const VGrid& vg__, const TS* __re
   const int64_t r0 = (int64_t)blockIdx.y * rows_per_chunk;
   const int64_t r1 = min(m, r0 + rows_per_chunk);
   const int ntile = r1 > r0 ? (int)((r1 - r0 + BR - 1) / BR) : 0;
-  const int t = threadIdx.x, wc = t >> 3, wa = t & 7;
+  const int t = threadIdx.x, cg4 = 4 * (t & 15), a4 = 4 * ((t >> 4) % (RP / 4)), rg = t / (4 * RP);
   auto issue = [&](int k) {
     const int64_t it = r0 + (int64_t)k * BR;
     TS* xs = Xs + (k % kWxStages) * XS;
@@ -1371,11 +1421,11 @@ __device__ __forceinline__ void wpass_mxp_body(const VGrid& vg__, const TS* __re
     }
     cp_async_commit();
   };
-  float acc[2][QA];
+  float acc[4][4];
 #pragma unroll
-  for (int x = 0; x < 2; ++x)
+  for (int x = 0; x < 4; ++x)
 #pragma unroll
-    for (int c = 0; c < QA; ++c) acc[x][c] = 0.f;
+    for (int c = 0; c < 4; ++c) acc[x][c] = 0.f;
   for (int k = 0; k < kWxStages - 1; ++k) {
     if (k < ntile) issue(k); else cp_async_commit();
   }
@@ -1386,40 +1436,37 @@ __device__ __forceinline__ void wpass_mxp_body(const VGrid& vg__, const TS* __re
     const TS* xs = Xs + (k % kWxStages) * XS;
     const float* us = Us + (k % kWxStages) * US;
 #pragma unroll 4
-    for (int ii = 0; ii < BR; ++ii) {
-      float x0, x1;
+    for (int ii = rg; ii < BR; ii += RS) {
+      float xv[4];
       if constexpr (std::is_same<TS, float>::value) {
-        const float2 w = *reinterpret_cast<const float2*>(xs + ii * BN + 2 * wc);
-        x0 = w.x; x1 = w.y;
+        const float4 w = *reinterpret_cast<const float4*>(xs + ii * BN + cg4);
+        xv[0] = w.x; xv[1] = w.y; xv[2] = w.z; xv[3] = w.w;
       } else {
-        const uint32_t w = *reinterpret_cast<const uint32_t*>(xs + ii * BN + 2 * wc);
-        x0 = __uint_as_float(w << 16); x1 = __uint_as_float(w & 0xFFFF0000u);
+        const uint2 w = *reinterpret_cast<const uint2*>(xs + ii * BN + cg4);
+        xv[0] = __uint_as_float(w.x << 16); xv[1] = __uint_as_float(w.x & 0xFFFF0000u);
+        xv[2] = __uint_as_float(w.y << 16); xv[3] = __uint_as_float(w.y & 0xFFFF0000u);
       }
-      float u[QA];
-      if constexpr (QA == 4) {
-        const float4 w = *reinterpret_cast<const float4*>(us + ii * RP + 4 * wa);
-        u[0] = w.x; u[1] = w.y; u[2] = w.z; u[3] = w.w;
-      } else if constexpr (QA == 2) {
-        const float2 w = *reinterpret_cast<const float2*>(us + ii * RP + 2 * wa);
-        u[0] = w.x; u[1] = w.y;
-      } else {
-        u[0] = us[ii * RP + wa];
-      }
+      const float4 u = *reinterpret_cast<const float4*>(us + ii * RP + a4);
+      const float uv[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
-      for (int c = 0; c < QA; ++c) {
-        acc[0][c] = fmaf(x0, u[c], acc[0][c]);
-        acc[1][c] = fmaf(x1, u[c], acc[1][c]);
-      }
+      for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[x][c] = fmaf(xv[x], uv[c], acc[x][c]);
     }
     __syncthreads();  // stage k % stages is refilled by the next iteration's issue
   }
   asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  __syncthreads();
+  float* part = reinterpret_cast<float*>(smem_raw);  // [RS][BN][RP] over the stages
 #pragma unroll
-  for (int x = 0; x < 2; ++x) {
-    const int64_t j = j0 + 2 * wc + x;
-    if (j < n)
+  for (int x = 0; x < 4; ++x)
+    *reinterpret_cast<float4*>(part + (rg * BN + cg4 + x) * RP + a4) = make_float4(acc[x][0], acc[x][1], acc[x][2], acc[x][3]);
+  __syncthreads();
+  for (int e = t; e < BN * RP; e += 256) {
+    float v = part[e];
 #pragma unroll
-      for (int c = 0; c < QA; ++c) Wpart[((int64_t)blockIdx.y * n + j) * RP + QA * wa + c] = acc[x][c];
+    for (int g = 1; g < RS; ++g) v += part[g * BN * RP + e];
+    if (j0 + e / RP < n) Wpart[((int64_t)blockIdx.y * n + j0) * RP + e] = v;
   }
 }
 
@@ -1721,9 +1768,16 @@ cudaError_t launch_reduce_parts(const double* parts, int count, int rpsq, double
 }
 
 cudaError_t launch_norm_m(const Shape& s, const Buffers& b, cudaStream_t st) {
-  const int blocks = (int)std::min<int64_t>(s.m, 1024);
+  const bool flat = b.m_dtype != SFR_F64 && s.ldm == s.n && reinterpret_cast<uintptr_t>(b.M) % 16 == 0;
+  const int blocks = (int)std::min<int64_t>(flat ? cdiv(s.m * s.n, 256 * 16) : s.m, 1024);
   cudaError_t e = by_mtype(b.m_dtype, b.M, [&](auto M) {
     using TMs = std::remove_const_t<std::remove_pointer_t<decltype(M)>>;
+    if constexpr (!std::is_same<TMs, double>::value) {
+      if (flat) {
+        launch_pdl(norm_flat_kernel<TMs>, blocks, 256, 0, st, M, s.m * s.n, b.normm_part);
+        return cudaGetLastError();
+      }
+    }
     launch_pdl(norm_m_kernel<TMs>, blocks, 256, 0, st, M, s.m, s.n, s.ldm, b.normm_part);
     return cudaGetLastError();
   });
@@ -1864,6 +1918,12 @@ cudaError_t launch_wpass(const Shape& s, const Buffers& b, bool fp64, bool first
         return f64_wpass(s, b, st);
       } else {
         if (std::is_same<TC, double>::value && !b.d_plain) return f64_wpass(s, b, st);
+        if constexpr (std::is_same<TC, float>::value && RP == 64) {
+          if (s.n % 4 == 0 && !b.tc)
+            return launch_k<&wpass_mxp_body<float, 64>, 256>(grid, 256, wxp_smem<float, 64>(), st,
+                                                             static_cast<const float*>(b.D), s.n, s.m, s.n,
+                                                             s.rows_per_chunk, U, Wp, b.st);
+        }
         launch_pdl(wpass_kernel<TC, TC, RP>, grid, 256, 0, st, static_cast<const TC*>(b.D), s.n, s.m, s.n, s.rows_per_chunk,
                    U, Wp, b.st);
         return cudaGetLastError();
@@ -1957,14 +2017,18 @@ cudaError_t launch_apply_v(const Shape& s, const Buffers& b, bool fp64, cudaStre
   });
 }
 
+// Mixed precision above rank 32 outside the tensor-core path (float32 M, or bfloat16 off its alignment rules): the
+// pipelined SIMT passes when their vector conditions hold (ldy = n here), else sweep_kernel / wpass_kernel.
+static bool mx64(const Shape& s, const Buffers& b, bool fp64) {
+  return !fp64 && s.rp == 64 && !b.tc && b.m_dtype != SFR_F64 && mx_vec(s, b);
+}
+
 static cudaError_t launch_sweep_mx(const Shape& s, const Buffers& b, int u_cur, cudaStream_t st) {
   dim3 grid(s.mx_grid_x, s.nsplit);
   const bool vec = mx_vec(s, b);
   return by_rank(s.rp, [&](auto rpc) {
     constexpr int RP = decltype(rpc)::value;
-    if constexpr (RP > 32) {
-      return cudaErrorInvalidValue;
-    } else {
+    {
       return by_mtype(b.m_dtype, b.M, [&](auto M) {
         using TMs = std::remove_const_t<std::remove_pointer_t<decltype(M)>>;
         auto go = [&](auto tag) {
@@ -1977,8 +2041,8 @@ static cudaError_t launch_sweep_mx(const Shape& s, const Buffers& b, int u_cur, 
         };
         if constexpr (!std::is_same<TMs, double>::value) {
           if (vec) {
-            if (g_recorder)
-              return launch_k<&sweep_mxp_any<TMs>, 256>(
+            if constexpr (RP <= 32)
+              if (g_recorder) return launch_k<&sweep_mxp_any<TMs>, 256>(
                   grid, 256, mxp_smem<TMs, 32>(64, 2), st, RP, M, s.m, s.n, s.ldm, b.ldy, static_cast<const float*>(b.Y[0]),
                   static_cast<float*>(b.Y[1]), static_cast<float*>(b.D), static_cast<const float*>(b.U[u_cur]),
                   static_cast<const float*>(b.C), static_cast<const float*>(b.V), static_cast<float*>(b.Qpart),
@@ -1997,7 +2061,10 @@ static cudaError_t launch_sweep_mx(const Shape& s, const Buffers& b, int u_cur, 
                 tw, nst, b.st);
           }
         }
-        return vec ? go(BodyTag<&sweep_mx_body<TMs, RP, true>>{}) : go(BodyTag<&sweep_mx_body<TMs, RP, false>>{});
+        if constexpr (RP <= 32)
+          return vec ? go(BodyTag<&sweep_mx_body<TMs, RP, true>>{}) : go(BodyTag<&sweep_mx_body<TMs, RP, false>>{});
+        else
+          return cudaErrorInvalidValue;
       });
     }
   });
@@ -2007,7 +2074,7 @@ cudaError_t launch_sweep(const Shape& s, const Buffers& b, bool fp64, int u_cur,
   // Y ping-pong: iteration k (0-based count of completed iterations) reads Y[k % 2] and writes
   // Y[(k + 1) % 2].  The host tracks k because graphs are replayed per iteration parity.
   if (fp64 && !b.plain) return f64_sweep(s, b, st);
-  if (mx_path(s, fp64)) return launch_sweep_mx(s, b, u_cur, st);
+  if (mx_path(s, fp64) || mx64(s, b, fp64)) return launch_sweep_mx(s, b, u_cur, st);
   // mixed precision above rank 32 outside the tensor-core path, and the plain float64 iterations
   dim3 grid(s.sweep_grid_x, s.nsplit);
   return by_prec(fp64, [&](auto tc) {
@@ -2037,7 +2104,7 @@ cudaError_t launch_sweep(const Shape& s, const Buffers& b, bool fp64, int u_cur,
 cudaError_t launch_iter_end(const Shape& s, const Buffers& b, bool fp64, cudaStream_t st) {
   // the mixed SIMT sweep writes one residual partial per (column split, 64-row block), the
   // float64 SIMT sweep one per 32-row block and split, the tensor-core sweep one per CTA
-  const int count = mx_path(s, fp64) ? s.nsplit * (int)((s.m + 63) / 64)
+  const int count = mx_path(s, fp64) || mx64(s, b, fp64) ? s.nsplit * (int)((s.m + 63) / 64)
                                      : (b.tc ? s.resid_parts : s.sweep_grid_x * s.nsplit);
   launch_k<&iter_end_body, 1024>(1, 1024, 0, st, b.resid_part, count, b.st);
   return cudaGetLastError();
