@@ -664,12 +664,6 @@ size_t wpass_smem(int r) {
   return 2 * 8 * (kBM * kTile + r4 * kLU) + kRed;
 }
 
-template <typename K>
-cudaError_t allow(K* kern, size_t smem) {
-  if (smem <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(reinterpret_cast<const void*>(kern), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-}
-
 }  // namespace
 
 // ---------------------------------------------------------------- launchers (called by sweep.cu's)
@@ -689,7 +683,7 @@ cudaError_t f64_gram(const Shape& s, const double* parts, int nparts, int64_t pa
   return by_rank(s.rp, [&](auto rpc) {
     auto kern = f64_gram_kernel<decltype(rpc)::value>;
     const size_t sm = gram_smem(s.rp, s.r, A != nullptr);
-    cudaError_t e = allow(kern, sm);
+    cudaError_t e = set_smem_attr<&f64_gram_kernel<decltype(rpc)::value>>(sm);
     if (e != cudaSuccess) return e;
     return launch_pdl(kern, ctas, kNT, sm, st, parts, nparts, part_stride, out, rows, A, H, gpart, s.r, dst);
   });
@@ -701,7 +695,7 @@ cudaError_t f64_transform(const Shape& s, const double* src, int64_t rows, int c
   return by_rank(s.rp, [&](auto rpc) {
     auto kern = f64_transform_kernel<decltype(rpc)::value>;
     const size_t sm = transform_smem(s.rp, s.r, hpart != nullptr, T2 != nullptr);
-    cudaError_t e = allow(kern, sm);
+    cudaError_t e = set_smem_attr<&f64_transform_kernel<decltype(rpc)::value>>(sm);
     if (e != cudaSuccess) return e;
     return launch_pdl(kern, ctas, kNT, sm, st, src, rows, T, dst, T2, dst2, old, hpart, static_cast<int2*>(F), eF,
                       static_cast<int2*>(F2), eF2, s.r, dstate);
@@ -716,7 +710,7 @@ cudaError_t f64_sweep(const Shape& s, const Buffers& b, cudaStream_t st) {
     auto go = [&](auto M) -> cudaError_t {
       using TMs = std::remove_const_t<std::remove_pointer_t<decltype(M)>>;
       auto kern = f64_sweep_kernel<TMs, decltype(rpc)::value>;
-      cudaError_t e = allow(kern, sm);
+      cudaError_t e = set_smem_attr<&f64_sweep_kernel<TMs, decltype(rpc)::value>>(sm);
       if (e != cudaSuccess) return e;
       return launch_pdl(kern, grid, kNT, sm, st, M, s.m, s.n, s.ldm, static_cast<const double*>(b.Y[0]),
                         static_cast<double*>(b.Y[1]), static_cast<int2*>(b.D), b.ldy, static_cast<const int2*>(b.P), b.ex,
@@ -733,7 +727,7 @@ cudaError_t f64_wpass(const Shape& s, const Buffers& b, cudaStream_t st) {
   const size_t sm = wpass_smem(s.r);
   return by_rank(s.rp, [&](auto rpc) {
     auto kern = f64_wpass_kernel<decltype(rpc)::value>;
-    cudaError_t e = allow(kern, sm);
+    cudaError_t e = set_smem_attr<&f64_wpass_kernel<decltype(rpc)::value>>(sm);
     if (e != cudaSuccess) return e;
     return launch_pdl(kern, dim3(s.wpass_grid_x, s.nchunk64), kNT, sm, st, static_cast<const int2*>(b.D), b.ldy, s.m, s.n,
                       s.rows_per_chunk64, static_cast<const int2*>(b.P), b.ex, static_cast<double*>(b.Wpart), s.r, b.st);

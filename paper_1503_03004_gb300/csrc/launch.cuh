@@ -148,13 +148,17 @@ inline int top_priority() {
   return v;
 }
 
-// Opts the kernel in to `smem` bytes of dynamic shared memory where static + dynamic exceed the
-// default 48 KB (a grouped kernel adds a few bytes of its own to the body's static use).
+// Opts the kernel in to all the dynamic shared memory its static use leaves of the 227 KB a CTA can have, where static +
+// dynamic exceed the default 48 KB (a grouped kernel adds a few bytes of its own to the body's static use).  The limit
+// belongs to the kernel, not to the launch: threads that launch it with different sizes must all set the same one, or
+// one lowers it between another's call here and its launch.
+constexpr int kSmemPerCta = 227 * 1024;
 template <auto Kern>
 cudaError_t set_smem_attr(size_t smem) {
-  if (smem == 0 || smem + static_smem<Kern>() <= 48 * 1024) return cudaSuccess;
+  const size_t fixed = static_smem<Kern>();
+  if (smem == 0 || smem + fixed <= 48 * 1024) return cudaSuccess;
   return cudaFuncSetAttribute(reinterpret_cast<const void*>(Kern), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)smem);
+                              kSmemPerCta - (int)fixed);
 }
 
 template <typename F> struct BodyTraits;
