@@ -35,13 +35,15 @@ __device__ __forceinline__ bool stopped(const DevState* st) { return *(volatile 
 // their fixed-order sum in the iteration end) do not depend on how many CTAs the sweep runs.  One
 // warp adds all 256 parts in float64: eight warps reducing their own with float64 shuffles took 40
 // float64 operations of the narrow pipe per row block, this takes 12.
+// (thread i's value at rs[(i / 4) ld + i % 4], ld = 4: an array.)
 template <typename TR>
 __device__ __forceinline__ void resid_store(const TR* rs, double* __restrict__ resid_part, int64_t split, int64_t nrb,
-                                            int64_t rb) {
+                                            int64_t rb, int ld = 4) {
   const int lane = threadIdx.x & 31;
-  double v = (double)rs[lane];
+  rs += (lane >> 2) * ld + (lane & 3);
+  double v = (double)rs[0];
 #pragma unroll
-  for (int w = 1; w < 8; ++w) v += (double)rs[lane + 32 * w];
+  for (int w = 1; w < 8; ++w) v += (double)rs[8 * w * ld];
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   if (lane == 0) resid_part[split * nrb + rb] = v;
 }
@@ -1017,15 +1019,20 @@ __device__ __forceinline__ void cp_async4(void* dst, const void* src, int src_by
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
 // The sweep above with every operand tile brought in by cp.async while earlier tiles are computed.
-// Pair k = the CTA's k-th (row block, column tile).  Y and M stand in a ring of `nst` stages of `tw`
-// columns (64, or n rounded up to 8 for narrow matrices, which leaves room for four stages: at n = 40 two stages kept
-// too few bytes in flight), U in a ring of row blocks, C in two buffers (transposed, its 4-column groups
-// XORed with the rank group, so that neither the 4-byte copies nor the 16-byte reads meet in a bank), V
-// in one, copied while the tile's L is formed.  X = L + Delta overwrites the Y tile.
+// Pair k = the CTA's k-th (row block, column tile).  Y and M of pair k + 1 are copied while pair k is computed (two
+// stages of `tw` columns: 64, or n rounded up to 8 for narrow matrices), V while the pair's L is formed, C (transposed,
+// its 4-column groups XORed with the rank group, so that neither the 4-byte copies nor the 16-byte reads meet in a
+// bank) and U of the next pair while Q is.  So C, U and V need one buffer each (with one column tile per row block:
+// two of U, copied with Y), which leaves room for a third CTA per SM on narrow matrices and a second one above rank
+// 32.  X = L + Delta overwrites the Y tile; the threads' residuals stand in its padding.
 // A thread's columns are 4 tc .. + 3 and 32 + 4 tc .. + 3, so that 8 threads read 128 contiguous bytes; sums over
 // ranks and columns run in order, 4 at a time from 16-byte reads (zeros past r and past the last column add nothing).
-// Loading the C and V tiles with plain loads after the barrier (the C stores 32 to a bank) used to take more than
-// half of each tile's time: 4096 x 2048, r = 32, bfloat16: 105 -> 60 us a sweep.
+// The kernel is bound by issue (60 % of the slots) and by the latency of its shared-memory reads, hence also: addresses
+// step from one base per tile, limits are 32-bit, and masks are left out where zeros do the same.
+// Per sweep: 4096 x 2048, r = 32, bfloat16 57 us (61 with masks and 64-bit addresses, 105 with plain loads of C and V
+// after the barrier); 2^20 x 40, r = 3, float32 133 us (186 with two CTAs per SM in four stages); 2048 x 2048, r = 40,
+// float32 65 us (98 with one CTA per SM).  4 x 4 outputs per thread in both products read a third less from shared
+// memory, but were slower (66, 222 and 121 us).
 // Needs the vector conditions (ldy % 4 == 0, 16-byte aligned rows of M) and float32 or bfloat16 M.
 template <typename TMs, int RP>
 __device__ __forceinline__ void sweep_mxp_body(const VGrid& vg__, const TMs* __restrict__ M, int64_t m, int64_t n, int64_t ldm,
@@ -1033,7 +1040,7 @@ __device__ __forceinline__ void sweep_mxp_body(const VGrid& vg__, const TMs* __r
                                                         float* __restrict__ D, const float* __restrict__ U,
                                                         const float* __restrict__ C, const float* __restrict__ V,
                                                         float* __restrict__ Qpart, int cols_per_split,
-                                                        double* __restrict__ resid_part, int r, int tw, int nst,
+                                                        double* __restrict__ resid_part, int r, int tw,
                                                         const DevState* st) {
   pdl_enter();
   SFR_VGRID(vg__);
@@ -1043,17 +1050,17 @@ __device__ __forceinline__ void sweep_mxp_body(const VGrid& vg__, const TMs* __r
   constexpr int QR = RP / 4;   // rank groups
   extern __shared__ __align__(16) unsigned char smem_raw[];
   using TR = std::conditional_t<RP == 64, double, float>;  // a thread's residual sum (above rank 32: float64 throughout)
-  __shared__ TR rs[256];
   const int ldx = tw + 4;
   const int64_t jbeg = (int64_t)blockIdx.y * cols_per_split;
   const int64_t jend = min(n, jbeg + cols_per_split);
   const int ntile = (int)((jend - jbeg + BN - 1) / BN);
-  const int nu = ntile == 1 ? nst : 2;
-  float* Ys = reinterpret_cast<float*>(smem_raw);                     // [nst][BM][ldx], then X
-  float* Us = Ys + nst * BM * ldx;                                    // [nu][BM][LDU]
-  float* Cs = Us + (nst > 2 ? nst : 2) * BM * LDU;                    // [2][RP][BN]
-  float* Vs = Cs + 2 * RP * BN;                                       // [BN][RP]
-  TMs* Ms = reinterpret_cast<TMs*>(Vs + BN * RP);                     // [nst][BM][tw]
+  const bool one = min(n, (int64_t)cols_per_split) <= BN;            // every row block is one pair
+  float* Ys = reinterpret_cast<float*>(smem_raw);                     // [2][BM][ldx], then X
+  float* Us = Ys + 2 * BM * ldx;                                      // [one ? 2 : 1][BM][LDU]
+  float* Vs = Us + (one ? 2 : 1) * BM * LDU;                          // [BN][RP]
+  TMs* Ms = reinterpret_cast<TMs*>(Vs + BN * RP);                     // [2][BM][tw]
+  float* Cs = reinterpret_cast<float*>(Ms + 2 * BM * tw);             // [r rounded up to 4][BN]
+  __shared__ double rs64[RP == 64 ? 256 : 1];
   const double mu_d = st->mu, mu_next = fmin(st->mu_max, st->rho * mu_d);
   const float mu = (float)mu_d, inv_mu = (float)(1.0 / mu_d), dcoef = (float)(1.0 / mu_d + 1.0 / mu_next);
   const int t = threadIdx.x, tr = t >> 3, tc = t & 7;
@@ -1062,96 +1069,109 @@ __device__ __forceinline__ void sweep_mxp_body(const VGrid& vg__, const TMs* __r
   const int64_t total = nmine * ntile;
 
   auto issue_v = [&](int64_t j0) {
-    for (int e = t; e < BN * QR; e += 256) {
-      const bool ok = j0 + e / QR < jend;
-      cp_async16(Vs + 4 * e, ok ? (const void*)(V + j0 * RP + 4 * e) : (const void*)V, ok ? 16 : 0);
+    const float* src = V + j0 * RP + 4 * t;
+    const int lim = (int)(jend - j0 < BN ? jend - j0 : BN) * QR;  // 16-byte chunks
+#pragma unroll
+    for (int e = t; e < BN * QR; e += 256, src += 1024) {
+      const bool ok = e < lim;
+      cp_async16(Vs + 4 * e, ok ? src : V, ok ? 16 : 0);
     }
   };
-  // the next pair to copy: row block, column tile, stage, U slot
-  int64_t irb = blockIdx.x;
-  int itile = 0, istage = 0, iu = 0, ic = 0;
-  auto issue = [&] {
-    const int64_t i0 = irb * BM, j0 = jbeg + (int64_t)itile * BN;
-    if (itile == 0) {
-      float* us = Us + iu * BM * LDU;
-      for (int e = t; e < BM * QR; e += 256) {
-        const int ii = e / QR, cc = e % QR;
-        const bool ok = i0 + ii < m;
-        cp_async16(us + ii * LDU + 4 * cc, ok ? (const void*)(U + (i0 + ii) * RP + 4 * cc) : (const void*)U, ok ? 16 : 0);
-      }
-    }
-    if (ntile > 1 || ic == 0) {  // C rows j0 + jj, rank 4 q + s -> Cs[4 q + s][jj]
-      float* cs = Cs + (ic & 1) * RP * BN;
-      ++ic;
+  // Addresses step by fixed strides from one base per tile and thread; row and column limits are 32-bit, and the
+  // tests drop out inside the matrix.
+  auto issue_u = [&](int64_t i0, float* us) {
+    const int lim = (int)(m - i0 < BM ? m - i0 : BM) * QR;  // 16-byte chunks
+    const float* src = U + i0 * RP + 4 * t;
 #pragma unroll
-      for (int it = 0; it < (RP == 64 ? 16 : RP == 32 ? 8 : 4); ++it) {
-        constexpr int JL = 32 / QR;  // columns a warp covers at a time
-        const int l = t & 31, q = l % QR, sI = it & 3;
-        const int jj = ((it >> 2) * 8 + (t >> 5)) * JL + l / QR, a = 4 * q + sI;
-        if (jj >= BN) continue;
-        const bool ok = j0 + jj < jend;
-        cp_async4(cs + a * BN + (((jj >> 2) ^ (q & 7)) << 2) + (jj & 3), ok ? (const void*)(C + (j0 + jj) * RP + a) : (const void*)C,
-                  ok ? 4 : 0);
-      }
+    for (int e = t; e < BM * QR; e += 256, src += 1024) {
+      const bool ok = e < lim;
+      cp_async16(us + (e / QR) * LDU + 4 * (e % QR), ok ? src : U, ok ? 16 : 0);
     }
-    float* ys = Ys + istage * BM * ldx;
-    {
-      const int cc = t & 15;  // 16-byte chunks of a row
-      const bool in = 4 * cc < tw, col = j0 + 4 * cc < jend;
+  };
+  auto issue_c = [&](int64_t j0) {  // C rows j0 + jj, rank 4 q + s -> Cs[4 q + s][jj]
+    const int cols = (int)(jend - j0 < BN ? jend - j0 : BN);
+    constexpr int JL = 32 / QR;  // columns a warp covers at a time
+    const int l = t & 31, q = l % QR, jb = (t >> 5) * JL + l / QR;
+    const float* src = C + (j0 + jb) * RP + 4 * q;
+    if (4 * q >= r) return;
 #pragma unroll
-      for (int it = 0; it < 4; ++it) {
-        const int ii = (t >> 4) + 16 * it;
-        const bool ok = col && i0 + ii < m;
-        if (in) cp_async16(ys + ii * ldx + 4 * cc, ok ? (const void*)(Yin + (i0 + ii) * ldy + j0 + 4 * cc) : (const void*)Yin, ok ? 16 : 0);
-      }
+    for (int it = 0; it < (RP == 64 ? 16 : RP == 32 ? 8 : 4); ++it) {
+      const int sI = it & 3, jj = jb + (it >> 2) * 8 * JL;
+      if (8 * JL > BN && jj >= BN) continue;
+      const bool ok = jj < cols;
+      cp_async4(Cs + (4 * q + sI) * BN + (((jj >> 2) ^ (q & 7)) << 2) + (jj & 3), ok ? src + (it >> 2) * 8 * JL * RP + sI : C,
+                ok ? 4 : 0);
     }
-    TMs* ms = Ms + istage * BM * tw;
-    {
-      constexpr int CPR = BN / EPC, RPI = 256 / CPR;
-      const int cc = t % CPR;
-      const bool in = EPC * cc < tw;
-      const int64_t left = jend - (j0 + EPC * cc);
-      const int bytes = left <= 0 ? 0 : (left >= EPC ? 16 : (int)left * (int)sizeof(TMs));
+  };
+  const int yc = 4 * (t & 15), yr = t >> 4;        // Y copies: rows yr + 16 it
+  constexpr int CPR = BN / EPC, RPI = 256 / CPR;   // M copies: rows mr + RPI it
+  const int mc = EPC * (t % CPR), mr = t / CPR;
+  const int64_t ystep = 16 * ldy, mstep = RPI * ldm;
+  auto issue_ym = [&](int64_t i0, int64_t j0, int istage) {
+    const int rows = (int)(m - i0 < BM ? m - i0 : BM), cols = (int)(jend - j0 < BN ? jend - j0 : BN);
+    float* yd = Ys + istage * BM * ldx + yr * ldx + yc;
+    const float* ysrc = Yin + (i0 + yr) * ldy + j0 + yc;
+    TMs* md = Ms + istage * BM * tw + mr * tw + mc;
+    const TMs* msrc = M + (i0 + mr) * ldm + j0 + mc;
+    if (rows == BM && cols == tw) {
+      if (yc < tw)
 #pragma unroll
-      for (int it = 0; it < BM / RPI; ++it) {
-        const int ii = t / CPR + RPI * it;
-        const bool ok = bytes > 0 && i0 + ii < m;
-        if (in) cp_async16(ms + ii * tw + EPC * cc, ok ? (const void*)(M + (i0 + ii) * ldm + j0 + EPC * cc) : (const void*)M, ok ? bytes : 0);
-      }
+        for (int it = 0; it < 4; ++it) cp_async16(yd + 16 * it * ldx, ysrc + it * ystep, 16);
+      if (mc < tw)
+#pragma unroll
+        for (int it = 0; it < BM / RPI; ++it) cp_async16(md + RPI * it * tw, msrc + it * mstep, 16);
+    } else {
+      if (yc < tw)
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {
+          const bool ok = yc < cols && yr + 16 * it < rows;
+          cp_async16(yd + 16 * it * ldx, ok ? ysrc + it * ystep : Yin, ok ? 16 : 0);
+        }
+      const int left = cols - mc, bytes = left <= 0 ? 0 : (left >= EPC ? 16 : left * (int)sizeof(TMs));
+      if (mc < tw)
+#pragma unroll
+        for (int it = 0; it < BM / RPI; ++it) {
+          const bool ok = bytes > 0 && mr + RPI * it < rows;
+          cp_async16(md + RPI * it * tw, ok ? msrc + it * mstep : M, ok ? bytes : 0);
+        }
     }
-    if (++itile == ntile) {
-      itile = 0;
-      irb += gridDim.x;
-      if (++iu == nu) iu = 0;
-    }
-    if (++istage == nst) istage = 0;
   };
 
-  if (ntile == 1 && total > 0) issue_v(jbeg);
-  for (int s = 0; s < nst - 1; ++s) {
-    if (s < total) issue();
-    cp_async_commit();
+  if (total > 0) {
+    const int64_t i0 = (int64_t)blockIdx.x * BM;
+    issue_ym(i0, jbeg, 0);
+    issue_u(i0, Us);
+    issue_c(jbeg);
+    if (ntile == 1) issue_v(jbeg);
   }
+  cp_async_commit();
   float q[2][QA];
   TR resid = 0;
   int64_t rb = blockIdx.x, rb_done = -1;
-  int tile = 0, stage = 0, cu = 0;
+  int tile = 0;
   for (int64_t k = 0; k < total; ++k) {
+    const int stage = (int)(k & 1);
     const int64_t i0 = rb * BM, j0 = jbeg + (int64_t)tile * BN;
-    if (nst == 2) cp_async_wait<0>();  // pair k has landed (this thread's copies)
-    else if (nst == 3) cp_async_wait<1>();
-    else cp_async_wait<2>();
-    __syncthreads();  // everyone's copies visible; the previous pair's readers are done
+    const bool last = tile == ntile - 1, more = k + 1 < total;
+    const int64_t i1 = last ? (rb + gridDim.x) * BM : i0, j1 = last ? jbeg : j0 + BN;  // pair k + 1
+    cp_async_wait<0>();  // pair k has landed (this thread's copies)
+    __syncthreads();     // everyone's copies visible; the previous pair's readers are done
     if (rb_done >= 0) {
-      if (t < 32) resid_store(rs, resid_part, blockIdx.y, nrb, rb_done);
+      if (t < 32) {
+        if constexpr (RP == 64) resid_store(rs64, resid_part, blockIdx.y, nrb, rb_done);
+        else resid_store(Ys + (stage ^ 1) * BM * ldx + tw, resid_part, blockIdx.y, nrb, rb_done, ldx);
+      }
       rb_done = -1;
     }
     if (ntile > 1) {
       issue_v(j0);
       cp_async_commit();
     }
-    if (k + nst - 1 < total) issue();
-    cp_async_commit();  // one group per iteration
+    if (more) {
+      issue_ym(i1, j1, stage ^ 1);
+      if (one) issue_u(i1, Us + (stage ^ 1) * BM * LDU);
+    }
+    cp_async_commit();
     if (tile == 0) {
 #pragma unroll
       for (int x = 0; x < 2; ++x)
@@ -1160,47 +1180,49 @@ __device__ __forceinline__ void sweep_mxp_body(const VGrid& vg__, const TMs* __r
       resid = 0;
     }
     // phase A: L for rows 2 tr, 2 tr + 1 and the thread's two column groups
-    const float* us = Us + cu * BM * LDU + 2 * tr * LDU;
-    const float* cs = Cs + (ntile > 1 ? (int)(k & 1) : 0) * RP * BN;
-    const bool two = tw > 32;
+    const float* us = Us + (one ? stage : 0) * BM * LDU + 2 * tr * LDU;
     float l[2][8];
 #pragma unroll
     for (int x = 0; x < 2; ++x)
 #pragma unroll
       for (int c = 0; c < 8; ++c) l[x][c] = 0.f;
+    auto form_l = [&](auto two) {
 #pragma unroll 2
-    for (int a4 = 0; a4 < r; a4 += 4) {
-      const float4 v0 = *reinterpret_cast<const float4*>(us + a4), v1 = *reinterpret_cast<const float4*>(us + LDU + a4);
-      const float u0[4] = {v0.x, v0.y, v0.z, v0.w}, u1[4] = {v1.x, v1.y, v1.z, v1.w};
-      const float* cp = cs + a4 * BN + ((tc ^ ((a4 >> 2) & 7)) << 2);
+      for (int a4 = 0; a4 < r; a4 += 4) {
+        const float4 v0 = *reinterpret_cast<const float4*>(us + a4), v1 = *reinterpret_cast<const float4*>(us + LDU + a4);
+        const float u0[4] = {v0.x, v0.y, v0.z, v0.w}, u1[4] = {v1.x, v1.y, v1.z, v1.w};
+        const float* cp = Cs + a4 * BN + ((tc ^ ((a4 >> 2) & 7)) << 2);
 #pragma unroll
-      for (int s4 = 0; s4 < 4; ++s4) {
-        const float4 c0 = *reinterpret_cast<const float4*>(cp + s4 * BN);
-        l[0][0] = fmaf(u0[s4], c0.x, l[0][0]); l[0][1] = fmaf(u0[s4], c0.y, l[0][1]);
-        l[0][2] = fmaf(u0[s4], c0.z, l[0][2]); l[0][3] = fmaf(u0[s4], c0.w, l[0][3]);
-        l[1][0] = fmaf(u1[s4], c0.x, l[1][0]); l[1][1] = fmaf(u1[s4], c0.y, l[1][1]);
-        l[1][2] = fmaf(u1[s4], c0.z, l[1][2]); l[1][3] = fmaf(u1[s4], c0.w, l[1][3]);
-        if (two) {
-          const float4 c1 = *reinterpret_cast<const float4*>(cp + s4 * BN + 32);
-          l[0][4] = fmaf(u0[s4], c1.x, l[0][4]); l[0][5] = fmaf(u0[s4], c1.y, l[0][5]);
-          l[0][6] = fmaf(u0[s4], c1.z, l[0][6]); l[0][7] = fmaf(u0[s4], c1.w, l[0][7]);
-          l[1][4] = fmaf(u1[s4], c1.x, l[1][4]); l[1][5] = fmaf(u1[s4], c1.y, l[1][5]);
-          l[1][6] = fmaf(u1[s4], c1.z, l[1][6]); l[1][7] = fmaf(u1[s4], c1.w, l[1][7]);
+        for (int s4 = 0; s4 < 4; ++s4) {
+          const float4 c0 = *reinterpret_cast<const float4*>(cp + s4 * BN);
+          l[0][0] = fmaf(u0[s4], c0.x, l[0][0]); l[0][1] = fmaf(u0[s4], c0.y, l[0][1]);
+          l[0][2] = fmaf(u0[s4], c0.z, l[0][2]); l[0][3] = fmaf(u0[s4], c0.w, l[0][3]);
+          l[1][0] = fmaf(u1[s4], c0.x, l[1][0]); l[1][1] = fmaf(u1[s4], c0.y, l[1][1]);
+          l[1][2] = fmaf(u1[s4], c0.z, l[1][2]); l[1][3] = fmaf(u1[s4], c0.w, l[1][3]);
+          if constexpr (decltype(two)::value) {
+            const float4 c1 = *reinterpret_cast<const float4*>(cp + s4 * BN + 32);
+            l[0][4] = fmaf(u0[s4], c1.x, l[0][4]); l[0][5] = fmaf(u0[s4], c1.y, l[0][5]);
+            l[0][6] = fmaf(u0[s4], c1.z, l[0][6]); l[0][7] = fmaf(u0[s4], c1.w, l[0][7]);
+            l[1][4] = fmaf(u1[s4], c1.x, l[1][4]); l[1][5] = fmaf(u1[s4], c1.y, l[1][5]);
+            l[1][6] = fmaf(u1[s4], c1.z, l[1][6]); l[1][7] = fmaf(u1[s4], c1.w, l[1][7]);
+          }
         }
       }
-    }
+    };
+    if (tw > 32) form_l(std::true_type{});
+    else form_l(std::false_type{});
     float* ys = Ys + stage * BM * ldx;
     const TMs* ms = Ms + stage * BM * tw;
+    // Outside the matrix M, Y and one factor of L are zeros, and so then are Y', Delta and X: no tests but at the stores.
+    const int rows = (int)(m - i0 < BM ? m - i0 : BM), cols = (int)(jend - j0 < BN ? jend - j0 : BN);
+    const int64_t out0 = (i0 + 2 * tr) * ldy + j0 + 4 * tc;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int c0 = 32 * h + 4 * tc;
       if (c0 >= tw) continue;
-      const int64_t jc = j0 + c0;
-      const int lim = (int)(jend - jc < 4 ? jend - jc : 4);  // valid columns (may be <= 0)
 #pragma unroll
       for (int x = 0; x < 2; ++x) {
         const int rr = 2 * tr + x;
-        const int64_t i = i0 + rr;
         const float4 yq = *reinterpret_cast<const float4*>(ys + rr * ldx + c0);
         const float yv[4] = {yq.x, yq.y, yq.z, yq.w};
         float mv[4];
@@ -1212,31 +1234,35 @@ __device__ __forceinline__ void sweep_mxp_body(const VGrid& vg__, const TMs* __r
           mv[0] = __uint_as_float(w.x << 16); mv[1] = __uint_as_float(w.x & 0xFFFF0000u);
           mv[2] = __uint_as_float(w.y << 16); mv[3] = __uint_as_float(w.y & 0xFFFF0000u);
         }
-        const bool row_ok = i < m;
         float yn[4], dd[4], xx[4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-          const bool ok = row_ok && c < lim;
           const float y = yv[c], lv = l[x][4 * h + c];
           const float z = mv[c] - lv + y * inv_mu;
           const float y1 = fminf(1.f, fmaxf(-1.f, mu * z));
           const float d = y1 * dcoef - y * inv_mu;
           const TR dy = y1 - y;
-          resid += ok ? dy * dy : (TR)0;
+          resid += dy * dy;
           yn[c] = y1;
           dd[c] = d;
-          xx[c] = ok ? lv + d : 0.f;  // X = L + Delta (0 outside the matrix)
+          xx[c] = lv + d;  // X = L + Delta
         }
         *reinterpret_cast<float4*>(ys + rr * ldx + c0) = make_float4(xx[0], xx[1], xx[2], xx[3]);
-        if (row_ok && lim > 0) {
-          *reinterpret_cast<float4*>(Yout + i * ldy + jc) = make_float4(yn[0], yn[1], yn[2], yn[3]);
-          *reinterpret_cast<float4*>(D + i * ldy + jc) = make_float4(dd[0], dd[1], dd[2], dd[3]);
+        if (rr < rows && c0 < cols) {
+          const int64_t o = out0 + (x ? ldy : 0) + 32 * h;
+          *reinterpret_cast<float4*>(Yout + o) = make_float4(yn[0], yn[1], yn[2], yn[3]);
+          *reinterpret_cast<float4*>(D + o) = make_float4(dd[0], dd[1], dd[2], dd[3]);
         }
       }
     }
     if (ntile > 1) cp_async_wait<1>();  // V of this tile
-    __syncthreads();                    // X (and V) complete
-    const int jn = (int)(jend - j0 < BN ? jend - j0 : BN);  // valid columns of the tile
+    __syncthreads();                    // X (and V) complete; U and C are free
+    if (more) {
+      if (ntile > 1) issue_c(j1);
+      if (!one && last) issue_u(i1, Us);
+    }
+    cp_async_commit();
+    const int jn = cols;
     const float* x0p = ys + 2 * tr * ldx;
     const float* vp = Vs + QA * tc;
 #pragma unroll 2
@@ -1266,7 +1292,7 @@ __device__ __forceinline__ void sweep_mxp_body(const VGrid& vg__, const TMs* __r
         }
       }
     }
-    if (tile == ntile - 1) {  // row block done: its Q partial and residual
+    if (last) {  // row block done: its Q partial and residual
 #pragma unroll
       for (int x = 0; x < 2; ++x) {
         const int64_t i = i0 + 2 * tr + x;
@@ -1274,25 +1300,27 @@ __device__ __forceinline__ void sweep_mxp_body(const VGrid& vg__, const TMs* __r
 #pragma unroll
           for (int c = 0; c < QA; ++c) Qpart[((int64_t)blockIdx.y * m + i) * RP + QA * tc + c] = q[x][c];
       }
-      rs[t] = resid;  // summed after the next barrier
+      if constexpr (RP == 64) rs64[t] = resid;  // summed after the next barrier
+      else ys[(t >> 2) * ldx + tw + (t & 3)] = resid;
       rb_done = rb;
     }
     if (++tile == ntile) {
       tile = 0;
       rb += gridDim.x;
-      if (++cu == nu) cu = 0;
     }
-    if (++stage == nst) stage = 0;
   }
   cp_async_wait<0>();
   __syncthreads();
-  if (rb_done >= 0 && t < 32) resid_store(rs, resid_part, blockIdx.y, nrb, rb_done);
+  if (rb_done >= 0 && t < 32) {
+    if constexpr (RP == 64) resid_store(rs64, resid_part, blockIdx.y, nrb, rb_done);
+    else resid_store(Ys + ((total - 1) & 1) * BM * ldx + tw, resid_part, blockIdx.y, nrb, rb_done, ldx);
+  }
 }
 
 template <typename TMs, int RP>
-constexpr size_t mxp_smem(int tw, int nst) {
-  return (size_t)nst * kMxBM * ((tw + 4) * 4 + tw * sizeof(TMs)) + (size_t)(nst > 2 ? nst : 2) * kMxBM * (RP + 4) * 4 +
-         (size_t)RP * 3 * kMxBN * 4;
+constexpr size_t mxp_smem(int tw, bool one, int r) {
+  return (size_t)2 * kMxBM * ((tw + 4) * 4 + tw * sizeof(TMs)) + (size_t)(one ? 2 : 1) * kMxBM * (RP + 4) * 4 +
+         (size_t)RP * kMxBN * 4 + (size_t)((r + 3) / 4 * 4) * kMxBN * 4;
 }
 
 // W pass, float32: Wpart[c][j][:] = sum over the rows i of chunk c of src[i][j] U[i][:].  CTA:
@@ -1656,7 +1684,7 @@ __device__ __forceinline__ void sweep_mxp_any(const VGrid& vg, int rp, const TMs
                                               const float* C, const float* V, float* Qpart, int cols_per_split,
                                               double* resid_part, int r, const DevState* st) {
   SFR_BY_RANK(rp, (sweep_mxp_body<TMs, RP>(vg, M, m, n, ldm, ldy, Yin, Yout, D, U, C, V, Qpart, cols_per_split, resid_part, r,
-                                           64, 2, st)));
+                                           64, st)));
 }
 template <typename TS>
 __device__ __forceinline__ void wpass_mxp_any(const VGrid& vg, int rp, const TS* src, int64_t lds, int64_t m, int64_t n,
@@ -1712,11 +1740,6 @@ size_t transform_smem() {
   // the Gram scratch (256 x 16) starts at the source-row tile, 2 RP (RP + 4) elements in
   return sizeof(TC) * std::max<size_t>((size_t)(2 * RP + 3 * kGramRows) * (RP + 4),
                                        (size_t)2 * RP * (RP + 4) + 16 * kThinThreads);
-}
-
-template <typename K>
-cudaError_t allow_smem(K kern, size_t bytes) {
-  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 }  // namespace
@@ -2043,22 +2066,17 @@ static cudaError_t launch_sweep_mx(const Shape& s, const Buffers& b, int u_cur, 
           if (vec) {
             if constexpr (RP <= 32)
               if (g_recorder) return launch_k<&sweep_mxp_any<TMs>, 256>(
-                  grid, 256, mxp_smem<TMs, 32>(64, 2), st, RP, M, s.m, s.n, s.ldm, b.ldy, static_cast<const float*>(b.Y[0]),
+                  grid, 256, mxp_smem<TMs, 32>(64, true, 32), st, RP, M, s.m, s.n, s.ldm, b.ldy, static_cast<const float*>(b.Y[0]),
                   static_cast<float*>(b.Y[1]), static_cast<float*>(b.D), static_cast<const float*>(b.U[u_cur]),
                   static_cast<const float*>(b.C), static_cast<const float*>(b.V), static_cast<float*>(b.Qpart),
                   s.cols_per_split, b.resid_part, s.r, b.st);
-            // narrow matrices: as many columns as needed and up to four stages in half an SM's shared memory
-            int tw = 64, nst = 2;
-            if (s.n <= 64) {
-              tw = (int)(s.n + 7) / 8 * 8;
-              while (nst < 4 && mxp_smem<TMs, RP>(tw, nst + 1) <= 110 * 1024) ++nst;
-            }
-            const size_t sm = mxp_smem<TMs, RP>(tw, nst);
+            const int tw = s.n <= 64 ? (int)(s.n + 7) / 8 * 8 : 64;  // narrow matrices: as many columns as needed
+            const size_t sm = mxp_smem<TMs, RP>(tw, std::min<int64_t>(s.n, s.cols_per_split) <= kMxBN, s.r);
             return launch_k<&sweep_mxp_body<TMs, RP>, 256>(
                 grid, 256, sm, st, M, s.m, s.n, s.ldm, b.ldy, static_cast<const float*>(b.Y[0]), static_cast<float*>(b.Y[1]),
                 static_cast<float*>(b.D), static_cast<const float*>(b.U[u_cur]), static_cast<const float*>(b.C),
                 static_cast<const float*>(b.V), static_cast<float*>(b.Qpart), s.cols_per_split, b.resid_part, s.r,
-                tw, nst, b.st);
+                tw, b.st);
           }
         }
         if constexpr (RP <= 32)
