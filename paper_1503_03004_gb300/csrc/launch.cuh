@@ -34,8 +34,13 @@ struct VGrid {
   (void)blockIdx;                    \
   (void)gridDim
 
+// The launch bounds NT are a number of threads, or per_sm(threads, CTAs) for a kernel whose registers have to leave room
+// for that many CTAs on an SM.
+constexpr int per_sm(int threads, int ctas) { return threads | ctas << 16; }
+#define SFR_BOUNDS(NT) __launch_bounds__((NT) & 0xFFFF, (NT) >> 16)
+
 template <auto Body, int NT, typename... T>
-__global__ void __launch_bounds__(NT) body_kernel(T... a) {
+__global__ void SFR_BOUNDS(NT) body_kernel(T... a) {
   Body(VGrid{blockIdx, gridDim}, a...);
 }
 
@@ -80,8 +85,8 @@ template <typename... T> struct GroupEntry {
 // [starts[p], starts[p + 1]).  The first warp finds p (starts ascending, count small), then the
 // body runs with the problem's own grid and arguments.
 template <auto Body, int NT, typename... T>
-__global__ void __launch_bounds__(NT) grouped_kernel(const int* __restrict__ starts,
-                                                     const GroupEntry<T...>* __restrict__ tab, int count) {
+__global__ void SFR_BOUNDS(NT) grouped_kernel(const int* __restrict__ starts,
+                                              const GroupEntry<T...>* __restrict__ tab, int count) {
   // the table was copied in after the previous kernel: wait for it as every body waits for its inputs
   asm volatile("griddepcontrol.wait;" ::: "memory");
   __shared__ int s_prob;

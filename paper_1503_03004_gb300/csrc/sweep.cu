@@ -281,6 +281,11 @@ __device__ __forceinline__ void load_rr(const double* __restrict__ g, TC* s, int
   }
 }
 
+// Registers of the float32 thin kernels: up to four CTAs per SM are launched on tall matrices, and with tiles of 2 or
+// 4 KB they are bound by the bytes in flight, so that all four have to fit up to rank 16 (2^20 rows, r = 3: Gram
+// 34.5 -> 25.2 us on average over both sides, with two resident before; loading four tiles ahead instead: 26.3 us).
+template <int RP> constexpr int kThinBounds = RP <= 16 ? per_sm(256, 4) : 256;
+
 // Elements of a kGramRows x RP row tile owned by thread t: e = t + q * 256, q < RP / 4.
 template <int RP>
 struct TileIdx {
@@ -1627,6 +1632,119 @@ __global__ void __launch_bounds__(256) finalize_kernel(const TMs* __restrict__ M
   if (L) L[i * lds + j] = (TSo)l;
 }
 
+// The same in float32 arithmetic, 64 x 128 outputs per CTA: a thread forms 4 rows x 8 columns, the sum over the ranks in
+// order, operands in 16-byte reads from shared memory; 16-byte accesses to M, Y, S and L where their rows allow
+// them (vec).  Bound by memory: 2^20 x 40, r = 3, float32 S and L 730 -> 235 us, 4096 x 2048, r = 32 106 -> 54 us
+// (one output per thread before, two shared-memory reads per multiply-add).
+constexpr int kFinRows = 64, kFinCols = 128, kFinK = 32;
+template <typename T>
+__device__ __forceinline__ void ld4(const T* p, float (&v)[4]) {
+  if constexpr (sizeof(T) == 2) {
+    const uint2 w = *reinterpret_cast<const uint2*>(p);
+    v[0] = __uint_as_float(w.x << 16); v[1] = __uint_as_float(w.x & 0xFFFF0000u);
+    v[2] = __uint_as_float(w.y << 16); v[3] = __uint_as_float(w.y & 0xFFFF0000u);
+  } else {
+    const float4 w = *reinterpret_cast<const float4*>(p);
+    v[0] = w.x; v[1] = w.y; v[2] = w.z; v[3] = w.w;
+  }
+}
+template <typename TMs, typename TSo, typename TY, int RP>
+__global__ void __launch_bounds__(256) finalize_f32_kernel(const TMs* __restrict__ M, int64_t m, int64_t n, int64_t ldm,
+                                                           const TY* __restrict__ Yprev, int64_t ldy,
+                                                           const float* __restrict__ U, const float* __restrict__ C,
+                                                           TSo* __restrict__ S, TSo* __restrict__ L, int64_t lds, int r,
+                                                           int vec, const DevState* st) {
+  pdl_enter();
+  __shared__ __align__(16) float us[kFinRows][kFinK + 4];
+  __shared__ __align__(16) float cs[kFinK][kFinCols + 4];
+  constexpr int KC = RP < kFinK ? RP : kFinK;
+  const int64_t nbx = (n + kFinCols - 1) / kFinCols;  // 1-D grid, columns fastest (a 2-D grid would cap m)
+  const int64_t i0 = ((int64_t)blockIdx.x / nbx) * kFinRows, j0 = ((int64_t)blockIdx.x % nbx) * kFinCols;
+  const int t = threadIdx.x, tc = t & 15, tr = t >> 4;  // rows tr + 16 x, columns 4 tc + 64 h + c
+  float l[4][8];
+#pragma unroll
+  for (int x = 0; x < 4; ++x)
+#pragma unroll
+    for (int c = 0; c < 8; ++c) l[x][c] = 0.f;
+  for (int k0 = 0; k0 < r; k0 += KC) {  // (U and C are zero in the ranks r .. RP)
+    const int k4 = min(KC, (r - k0 + 3) & ~3);
+    __syncthreads();
+    for (int e = t; e < kFinRows * KC; e += 256) {
+      const int ii = e / KC, a = e % KC;
+      us[ii][a] = i0 + ii < m ? U[(i0 + ii) * RP + k0 + a] : 0.f;
+    }
+    for (int e = t; e < kFinCols * KC; e += 256) {
+      const int jj = e / KC, a = e % KC;
+      cs[a][jj] = j0 + jj < n ? C[(j0 + jj) * RP + k0 + a] : 0.f;
+    }
+    __syncthreads();
+    for (int a4 = 0; a4 < k4; a4 += 4) {
+      float u[4][4];
+#pragma unroll
+      for (int x = 0; x < 4; ++x) ld4(&us[tr + 16 * x][a4], u[x]);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        float v0[4], v1[4];
+        ld4(&cs[a4 + q][4 * tc], v0);
+        ld4(&cs[a4 + q][64 + 4 * tc], v1);
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            l[x][c] = fmaf(u[x][q], v0[c], l[x][c]);
+            l[x][4 + c] = fmaf(u[x][q], v1[c], l[x][4 + c]);
+          }
+      }
+    }
+  }
+  const float inv_mu = (float)(1.0 / st->mu_last);
+#pragma unroll
+  for (int x = 0; x < 4; ++x) {
+    const int64_t i = i0 + tr + 16 * x;
+    if (i >= m) continue;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int64_t j = j0 + 64 * h + 4 * tc;
+      if (j >= n) continue;
+      const float* lv = l[x] + 4 * h;
+      const bool in4 = j + 4 <= n;
+      float mv[4] = {0.f, 0.f, 0.f, 0.f}, yv[4] = {0.f, 0.f, 0.f, 0.f}, sv[4];
+      if constexpr (sizeof(TMs) <= 4) {
+        if (in4 && (vec & 2)) ld4(M + i * ldm + j, mv);
+      }
+      if (!(in4 && (vec & 2) && sizeof(TMs) <= 4))
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (j + c < n) mv[c] = ld_as<float, TMs>(M + i * ldm + j + c);
+      if (in4 && (vec & 4)) {
+        ld4(Yprev + i * ldy + j, yv);
+      } else {
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (j + c < n) yv[c] = ld_as<float, TY>(Yprev + i * ldy + j + c);
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float z = mv[c] - lv[c] + yv[c] * inv_mu;
+        sv[c] = z > inv_mu ? z - inv_mu : (z < -inv_mu ? z + inv_mu : 0.f);
+      }
+      if constexpr (sizeof(TSo) == 4) {
+        if (in4 && (vec & 1)) {
+          if (S) *reinterpret_cast<float4*>(S + i * lds + j) = make_float4(sv[0], sv[1], sv[2], sv[3]);
+          if (L) *reinterpret_cast<float4*>(L + i * lds + j) = make_float4(lv[0], lv[1], lv[2], lv[3]);
+          continue;
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (j + c < n) {
+          if (S) S[i * lds + j + c] = (TSo)sv[c];
+          if (L) L[i * lds + j + c] = (TSo)lv[c];
+        }
+    }
+  }
+}
+
 template <typename TC, int RP>
 __global__ void export_kernel(const TC* __restrict__ src, int64_t rows, int r, double* __restrict__ dst) {
   pdl_enter();
@@ -1840,7 +1958,7 @@ cudaError_t launch_gram_p(const Shape& s, const Buffers& b, bool fp64, bool sum_
   return by_rank(s.rp, [&](auto rpc) {
     constexpr int RP = decltype(rpc)::value;
     const size_t sm = gram_smem<float, RP>();
-    launch_k<&thin_gram_body<float, RP>, 256>(s.gp_blocks, 256, sm, st,
+    launch_k<&thin_gram_body<float, RP>, kThinBounds<RP>>(s.gp_blocks, 256, sm, st,
         static_cast<const float*>(b.Qpart), sum_parts ? s.nsplit : 0, s.m * RP, static_cast<float*>(b.P), s.m,
         static_cast<const float*>(addA), H, b.GPpart, b.st, s.q_ctas, (s.n + 63) / 64, (const double*)nullptr,
         pt ? static_cast<__nv_bfloat16*>(b.t.Ut) : nullptr, (int64_t)b.t.ldd);
@@ -1874,7 +1992,7 @@ cudaError_t launch_apply_u(const Shape& s, const Buffers& b, bool fp64, bool fir
     // W pass, its bfloat16 transpose (later W passes take P^T from the P / Gram kernel)
     // (Algorithm 4: the two-term bfloat16 split of U^T instead, the B operand of M^T U)
     const bool tcx = b.tc && RP == 64, tf = tcx && !b.full;
-    launch_k<&row_transform_body<float, RP>, 256>(s.gp_blocks, 256, sm, st,
+    launch_k<&row_transform_body<float, RP>, kThinBounds<RP>>(s.gp_blocks, 256, sm, st,
         static_cast<const float*>(b.P), s.m, b.TU, static_cast<float*>(b.U[u_new]), nullptr, nullptr,
         first ? nullptr : static_cast<const float*>(b.U[u_old]), first ? nullptr : b.Hpart, b.st,
         tf ? b.t.Uh : nullptr, tf ? b.t.Ul : nullptr,
@@ -1999,7 +2117,7 @@ cudaError_t launch_wfinal(const Shape& s, const Buffers& b, bool fp64, bool firs
   return by_rank(s.rp, [&](auto rpc) {
     constexpr int RP = decltype(rpc)::value;
     const size_t sm = gram_smem<float, RP>();
-    launch_k<&thin_gram_body<float, RP>, 256>(s.gw_blocks, 256, sm, st,
+    launch_k<&thin_gram_body<float, RP>, kThinBounds<RP>>(s.gw_blocks, 256, sm, st,
         static_cast<const float*>(b.Wpart), nparts, s.n * RP, static_cast<float*>(b.W), s.n,
         first ? nullptr : static_cast<const float*>(b.C), first ? nullptr : H, b.GWpart, b.st, 0, (int64_t)0,
         wp ? (const double*)b.TU : (const double*)nullptr, (__nv_bfloat16*)nullptr, (int64_t)0);
@@ -2032,7 +2150,7 @@ cudaError_t launch_apply_v(const Shape& s, const Buffers& b, bool fp64, cudaStre
     // tensor-core path: also the TF32 split of C and the bfloat16 transpose of V
     // (Algorithm 4: the two-term bfloat16 split of V^T instead, the B operand of M V)
     const bool tcx = b.tc && RP == 64, tf = tcx && !b.full;
-    launch_k<&row_transform_body<float, RP>, 256>(s.gw_blocks, 256, sm, st,
+    launch_k<&row_transform_body<float, RP>, kThinBounds<RP>>(s.gw_blocks, 256, sm, st,
         static_cast<const float*>(b.W), s.n, b.TV, static_cast<float*>(b.V), b.TCm, static_cast<float*>(b.C), nullptr, nullptr,
         b.st, tf ? b.t.Ch : nullptr, tf ? b.t.Cl : nullptr, tcx ? static_cast<__nv_bfloat16*>(b.t.Vt) : nullptr,
         (int64_t)b.t.ldy, b.full ? 1 : 0);
@@ -2133,7 +2251,6 @@ cudaError_t launch_finalize(const Shape& s, const Buffers& b, bool fp64, int u_c
   // Y_prev is the multiplier the last sweep read: Buffers::Y[0] by the host's swap convention.
   const int64_t nblk = (int64_t)cdiv(s.n, 32) * cdiv(s.m, 8);
   if (nblk > 0x7fffffffLL) return cudaErrorInvalidValue;
-  const unsigned grid = (unsigned)nblk;
   return by_prec(fp64, [&](auto tc) {
     using TC = decltype(tc);
     return by_rank(s.rp, [&](auto rpc) {
@@ -2142,14 +2259,24 @@ cudaError_t launch_finalize(const Shape& s, const Buffers& b, bool fp64, int u_c
         using TMs = std::remove_const_t<std::remove_pointer_t<decltype(M)>>;
         auto go = [&](auto yptr, int64_t ldy) {
           using TY = std::remove_const_t<std::remove_pointer_t<decltype(yptr)>>;
-          if (s_dtype == SFR_F64)
-            launch_pdl(finalize_kernel<TC, TMs, double, TY, RP>, grid, 256, 0, st,
-                M, s.m, s.n, s.ldm, yptr, ldy, static_cast<const TC*>(b.U[u_cur]), static_cast<const TC*>(b.C),
-                static_cast<double*>(S), static_cast<double*>(L), lds, b.st);
-          else
-            launch_pdl(finalize_kernel<TC, TMs, float, TY, RP>, grid, 256, 0, st,
-                M, s.m, s.n, s.ldm, yptr, ldy, static_cast<const TC*>(b.U[u_cur]), static_cast<const TC*>(b.C),
-                static_cast<float*>(S), static_cast<float*>(L), lds, b.st);
+          auto out = [&](auto so) {
+            using TSo = decltype(so);
+            TSo *Sp = static_cast<TSo*>(S), *Lp = static_cast<TSo*>(L);
+            if constexpr (std::is_same<TC, double>::value) {
+              launch_pdl(finalize_kernel<TC, TMs, TSo, TY, RP>, (unsigned)nblk, 256, 0, st, M, s.m, s.n, s.ldm, yptr, ldy,
+                         static_cast<const double*>(b.U[u_cur]), static_cast<const double*>(b.C), Sp, Lp, lds, b.st);
+            } else {
+              // bit 0: 16-byte stores to S and L, bit 1: loads of 4 elements of M, bit 2: of Y
+              const int vec = (sizeof(TSo) == 4 && (uintptr_t)S % 16 == 0 && (uintptr_t)L % 16 == 0 && lds % 4 == 0 ? 1 : 0) |
+                              (sizeof(TMs) <= 4 && (uintptr_t)M % 16 == 0 && s.ldm % 4 == 0 ? 2 : 0) |
+                              ((uintptr_t)yptr % 16 == 0 && ldy % 4 == 0 ? 4 : 0);
+              launch_pdl(finalize_f32_kernel<TMs, TSo, TY, RP>, cdiv(s.n, kFinCols) * cdiv(s.m, kFinRows), 256, 0, st, M,
+                         s.m, s.n, s.ldm, yptr, ldy, static_cast<const float*>(b.U[u_cur]), static_cast<const float*>(b.C),
+                         Sp, Lp, lds, s.r, vec, b.st);
+            }
+          };
+          if (s_dtype == SFR_F64) out(double{});
+          else out(float{});
           return cudaGetLastError();
         };
         if (b.tc) return go(static_cast<const __nv_bfloat16*>(b.Y[0]), b.t.ldy);
