@@ -196,15 +196,17 @@ constexpr int kGramRows = 64;    // rows per Gram / transform CTA
 // Float64 solves of rank above 16 run their first iterations with float64 multiply-add loops (sweep.cu's
 // kernels) and switch to the fixed-point products of f64.cu after kPlainIters.  In those iterations the
 // projector starts far from its previous eigenbasis and corrects it in float32: a last-bit change of a
-// Gram matrix then turns U, B and V together by up to 1e-9 (L and S stay within 1e-13), where later it
-// moves them by 1e-14, so keeping the arithmetic of the start keeps the factors reproducible.  Turned
-// by, over 20 inputs each, without a plain start: 2.5e-10 at 500 x 500, r = 25, 6.4e-10 at 300 x 260, r = 32, 1e-9 at 4096 x
-// 4096, r = 64, but 1.4e-11 at r = 10; with it 3e-13 at r = 64.  kPlainIters + 1 is odd: the buffers alternate every iteration.
+// Gram matrix then turns U, B and V together (L and S stay within 1e-13), where later it mostly moves them by
+// 1e-14.  Turned against plain iterations throughout: without a plain start 2.5e-10 at 500 x 500, r = 25,
+// 6.4e-10 at 300 x 260, r = 32, 1e-9 at 4096 x 4096, r = 64, but 1.4e-11 at r = 10 (20 inputs each); with it 1e-13 at
+// the median and 4e-10 at worst (49 inputs, r = 25-64; the few above 1e-12 had a cold call later on: 10 plain
+// iterations leave 4e-10 too, and each costs 4 ms at 4096 x 4096).  kPlainIters + 1 is odd: the buffers alternate.
 constexpr int kPlainIters = 6;
 inline bool plain_start(int rp, bool fp64) { return fp64 && rp > 16; }
 
 inline int pad_rank(int r) { return r <= 8 ? 8 : r <= 16 ? 16 : r <= 32 ? 32 : 64; }
-// The mixed path's float32 SIMT passes for r <= 32 (sweep_mx*/wpass_mx* kernels).
+// The mixed path's float32 SIMT passes for r <= 32 (sweep_mx*/wpass_mx* kernels), whatever the alignment of M; above,
+// launch_sweep takes the pipelined ones where M's rows allow it.
 inline bool mx_path(const Shape& s, bool fp64) { return !fp64 && s.rp <= 32; }
 // Leading dimension of the aligned copy of M that the SIMT mixed passes read when the caller's rows
 // are not 16-byte aligned (0: no copy; the tensor-core path has its own alignment rule).

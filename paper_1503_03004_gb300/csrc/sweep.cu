@@ -1,6 +1,7 @@
 // m x n and thin (m x r, n x r) kernels of one FR-ADM iteration (Algorithm 1 with
-// the L-step of Algorithm 3), SIMT version for float64 (FP64 path) and float32
-// (mixed path) arithmetic.
+// the L-step of Algorithm 3), SIMT version: the mixed path's float32 arithmetic off the
+// tensor cores, and float64 multiply-add for Algorithm 4 and the plain first iterations of
+// a float64 solve (its other iterations run f64.cu's kernels).
 //
 // Notation (Algorithm 1): X_k = M - S_k + Y_k / mu_k, the matrix handed to
 // FixedRankOptStep.  The L-step computes
@@ -799,9 +800,9 @@ __global__ void __launch_bounds__(256) sweep_kernel(const TMs* __restrict__ M, i
   if (t == 0) resid_part[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = resid;
 }
 
-// ---------------------------------------------------------------- mixed-path SIMT passes (r <= 32)
+// ---------------------------------------------------------------- mixed-path SIMT passes
 // Float32 versions of the sweep and the W pass for the mixed path when the tensor-core kernels do
-// not apply (r <= 32, or M not bfloat16).  The work per element is small (2 r FMAs in the sweep,
+// not apply (r <= 32, or M not bfloat16, or off their alignment).  The work per element is small (2 r FMAs in the sweep,
 // r in the W pass), so these are built for bandwidth: 128-bit loads and stores along rows, L and
 // the thin products register-blocked (2 x 8 and 2 x r/8 per thread) so that shared-memory
 // operands are mostly broadcasts, and CTAs that loop over row blocks (the C / V tile stays
@@ -1414,9 +1415,8 @@ __device__ __forceinline__ void wpass_mx_body(const VGrid& vg__, const TS* __res
 // The W pass above with cp.async staging: 32-row tiles of src and U in a 4-stage ring, three
 // tiles in flight while one is accumulated.  A thread forms 4 columns x 4 ranks from 16-byte reads (two per 16
 // multiply-adds; 2 columns x r/8 ranks took two per 2 to 8) over every RS-th row of a tile, RS = 64 / RP row
-// groups, whose sums are added through shared memory at the end: 2^20 x 40, r = 3 101 -> 66 us, 2048 x 2048, r = 40
-// 45 -> 27 us.  Needs the vector conditions (src rows 16-byte
-// aligned, n % 4 == 0) and float32 or bfloat16 src.
+// groups, whose sums are added through shared memory at the end: 2^20 x 40, r = 3 101 -> 64 us, 2048 x 2048, r = 40
+// 45 -> 27 us.  Needs the vector conditions (src rows 16-byte aligned, n % 4 == 0) and float32 or bfloat16 src.
 constexpr int kWxStages = 4;
 template <typename TS, int RP>
 __device__ __forceinline__ void wpass_mxp_body(const VGrid& vg__, const TS* __restrict__ src, int64_t lds, int64_t m, int64_t n,
@@ -1862,8 +1862,8 @@ size_t transform_smem() {
 
 }  // namespace
 
-// Mixed path, r <= 32: the float32 passes above.  Vector loads need n % 4 == 0 and M rows on
-// 16-byte boundaries; otherwise the same kernels load element by element.
+// The float32 passes above: vector loads and copies need a leading dimension of Y that is a multiple of 4 and M rows on
+// 16-byte boundaries.  Otherwise r <= 32 loads element by element, and above sweep_kernel / wpass_kernel run.
 static bool mx_vec(const Shape& s, const Buffers& b) {
   const size_t es = b.m_dtype == SFR_F64 ? 8 : b.m_dtype == SFR_F32 ? 4 : 2;
   return b.ldy % 4 == 0 && ((size_t)s.ldm * es) % 16 == 0 && (reinterpret_cast<uintptr_t>(b.M) % 16) == 0;
@@ -2159,7 +2159,8 @@ cudaError_t launch_apply_v(const Shape& s, const Buffers& b, bool fp64, cudaStre
 }
 
 // Mixed precision above rank 32 outside the tensor-core path (float32 M, or bfloat16 off its alignment rules): the
-// pipelined SIMT passes when their vector conditions hold (ldy = n here), else sweep_kernel / wpass_kernel.
+// pipelined SIMT passes when their vector conditions hold (ldy = n here), else sweep_kernel / wpass_kernel
+// (2048 x 2048, r = 40, float32: sweep 74 -> 65 us, W pass 50 -> 27 us).
 static bool mx64(const Shape& s, const Buffers& b, bool fp64) {
   return !fp64 && s.rp == 64 && !b.tc && b.m_dtype != SFR_F64 && mx_vec(s, b);
 }
