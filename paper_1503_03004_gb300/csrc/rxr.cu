@@ -100,9 +100,10 @@ __device__ __noinline__ void mm_dist(const double* A, const TB* B, TCo* C, int r
   cg::cluster_group cl = cg::this_cluster();
   const int cs = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int rpc = (r + cs - 1) / cs, i0 = min(r, rank * rpc), i1 = min(r, i0 + rpc);
-  for (int e = threadIdx.x; e < (i1 - i0) * DM::RP; e += DM::NT) {
-    const int i = i0 + e / DM::RP, j = e % DM::RP;
-    if (j >= r) continue;
+  // (packed in r, not RP: a warp with idle lanes takes the float64 pipe as long as a full one:
+  // r = 5 23.6 -> 21.7 us a call, r = 10 34.5 -> 31.7)
+  for (int e = threadIdx.x; e < (i1 - i0) * r; e += DM::NT) {
+    const int i = i0 + e / r, j = e % r;
     // four independent chains (k mod 4) keep the float64 pipe busy with few warps per SM
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
     int k = 0;
