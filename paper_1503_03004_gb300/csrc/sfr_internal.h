@@ -137,7 +137,8 @@ struct Buffers {
   DevState* st;
   int u_cur;            // which U buffer holds the current U_bar (host-side bookkeeping)
   bool tc;              // tensor-core path (mixed precision, r <= 64, bfloat16 M)
-  bool plain;           // float64 path: this iteration's products are float64 loops (kPlainIters)
+  bool plain;           // float64 path: this iteration's products are float64 loops (kPlainIters; Algorithm 4 always:
+                        // its two passes over M bound it, and it starts with cold projector calls)
   bool d_plain;         // D holds float64 values (the last sweep was a plain one)
   bool full;            // Algorithm 4 on a fixed M: no multiplier or Delta buffers; the
                         // tensor-core path keeps two-term bfloat16 splits of U^T and V^T

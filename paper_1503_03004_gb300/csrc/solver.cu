@@ -783,6 +783,7 @@ struct Solver {
     b.M = Mdev;
     b.m_dtype = p.m_dtype;
     b.u_cur = 0;
+    b.plain = fp64;  // float64 products throughout (Buffers::plain)
 
     DevState h{};
     h.tol = p.tol;

@@ -1823,7 +1823,7 @@ cudaError_t by_rank(int rp, F&& f) {
   }
 }
 
-// Padded ranks whose float64 solves start with plain iterations (plain_start).
+// Padded ranks whose float64 FR-ADM solves start with plain iterations (plain_start).
 template <typename F>
 cudaError_t by_plain_rank(int rp, F&& f) {
   switch (rp) {
@@ -1944,7 +1944,7 @@ cudaError_t launch_gram_p(const Shape& s, const Buffers& b, bool fp64, bool sum_
     return f64_gram(s, static_cast<const double*>(b.Qpart), sum_parts ? s.nsplit : 0, s.m * s.rp,
                     static_cast<double*>(b.P), s.m, s.gp_blocks, static_cast<const double*>(addA), H, b.GPpart, b.st, st);
   if (fp64)
-    return by_plain_rank(s.rp, [&](auto rpc) {
+    return by_rank(s.rp, [&](auto rpc) {
       constexpr int RP = decltype(rpc)::value;
       return launch_k<&thin_gram_body<double, RP>, 256>(s.gp_blocks, 256, gram_smem<double, RP>(), st,
           static_cast<const double*>(b.Qpart), sum_parts ? s.nsplit : 0, s.m * RP, static_cast<double*>(b.P), s.m,
@@ -1970,7 +1970,7 @@ cudaError_t launch_apply_u(const Shape& s, const Buffers& b, bool fp64, bool fir
   // U_new = P T_U into the other U buffer; H partials U_old^T U_new (iteration >= 2).
   const int u_old = b.u_cur, u_new = 1 - b.u_cur;
   if (fp64 && b.plain)
-    return by_plain_rank(s.rp, [&](auto rpc) {
+    return by_rank(s.rp, [&](auto rpc) {
       constexpr int RP = decltype(rpc)::value;
       return launch_k<&row_transform_body<double, RP>, 256>(s.gp_blocks, 256, transform_smem<double, RP>(), st,
           static_cast<const double*>(b.P), s.m, b.TU, static_cast<double*>(b.U[u_new]), (const double*)nullptr,
@@ -1980,7 +1980,7 @@ cudaError_t launch_apply_u(const Shape& s, const Buffers& b, bool fp64, bool fir
   if (fp64)
     return f64_transform(s, static_cast<const double*>(b.P), s.m, s.gp_blocks, b.TU, static_cast<double*>(b.U[u_new]),
                          nullptr, nullptr, first ? nullptr : static_cast<const double*>(b.U[u_old]),
-                         first ? nullptr : b.Hpart, b.full ? nullptr : b.P, b.ex, nullptr, nullptr, b.st, st);
+                         first ? nullptr : b.Hpart, b.P, b.ex, nullptr, nullptr, b.st, st);
   if (g_recorder && s.rp <= 32)
     return launch_k<&row_transform_any, 256>(s.gp_blocks, 256, transform_smem<float, 32>(), st, s.rp,
         static_cast<const float*>(b.P), s.m, b.TU, static_cast<float*>(b.U[u_new]), (const double*)nullptr, (float*)nullptr,
@@ -2099,7 +2099,7 @@ cudaError_t launch_wfinal(const Shape& s, const Buffers& b, bool fp64, bool firs
     nparts = 1;
   }
   if (fp64 && b.plain)
-    return by_plain_rank(s.rp, [&](auto rpc) {
+    return by_rank(s.rp, [&](auto rpc) {
       constexpr int RP = decltype(rpc)::value;
       return launch_k<&thin_gram_body<double, RP>, 256>(s.gw_blocks, 256, gram_smem<double, RP>(), st,
           static_cast<const double*>(b.Wpart), nparts, s.n * RP, static_cast<double*>(b.W), s.n,
@@ -2127,7 +2127,7 @@ cudaError_t launch_wfinal(const Shape& s, const Buffers& b, bool fp64, bool firs
 
 cudaError_t launch_apply_v(const Shape& s, const Buffers& b, bool fp64, cudaStream_t st) {
   if (fp64 && b.plain)
-    return by_plain_rank(s.rp, [&](auto rpc) {
+    return by_rank(s.rp, [&](auto rpc) {
       constexpr int RP = decltype(rpc)::value;
       return launch_k<&row_transform_body<double, RP>, 256>(s.gw_blocks, 256, transform_smem<double, RP>(), st,
           static_cast<const double*>(b.W), s.n, b.TV, static_cast<double*>(b.V), b.TCm, static_cast<double*>(b.C),
@@ -2137,8 +2137,8 @@ cudaError_t launch_apply_v(const Shape& s, const Buffers& b, bool fp64, cudaStre
   if (fp64) {
     const int64_t tu = (s.m + kGramRows - 1) / kGramRows, tv = (s.n + kGramRows - 1) / kGramRows;
     return f64_transform(s, static_cast<const double*>(b.W), s.n, s.gw_blocks, b.TV, static_cast<double*>(b.V), b.TCm,
-                         static_cast<double*>(b.C), nullptr, nullptr, b.full ? nullptr : b.W, b.ex + tu + tv,
-                         b.full ? nullptr : b.Wpart, b.ex + tu, b.st, st);
+                         static_cast<double*>(b.C), nullptr, nullptr, b.W, b.ex + tu + tv, b.Wpart, b.ex + tu,
+                         b.st, st);
   }
   if (g_recorder && s.rp <= 32)
     return launch_k<&row_transform_any, 256>(s.gw_blocks, 256, transform_smem<float, 32>(), st, s.rp,
