@@ -6,7 +6,7 @@
 // integer slices whose products are accumulated exactly (the Ozaki scheme: Ozaki, Ogita, Oishi and
 // Rump, "Error-free transformations of matrix multiplication", Numer. Algorithms 59, 2012; here two
 // 28-bit slices and 64-bit integer accumulators instead of short floating-point slices):
-//   * a block of an operand shares one exponent e, with |x| < 2^e for all its entries;
+//   * the entries of an operand that meet in one sum share one exponent e, with |x| < 2^e for all of them;
 //   * x 2^(56-e) is rounded to an integer F, |F| <= 2^56, held as F = hi 2^28 + lo with
 //     |hi| <= 2^28, -2^27 <= lo < 2^27;
 //   * x y 2^(112 - e_x - e_y) = hi hi' 2^56 + (hi lo' + lo hi') 2^28 + lo lo', and the last term,
@@ -14,8 +14,14 @@
 // Sums over at most kTerms = 64 products cannot overflow (64 2^56 = 2^62, 128 2^55 = 2^62), and they
 // are exact, so they do not depend on the order of the terms.  Errors per product, relative to the
 // bound 2^(e_x + e_y): 2^-57 for each operand's rounding and 2^-58 for the dropped term, against
-// 2^-54 for the rounding of a float64 operation at that size: the fixed-point sum is at least as
-// accurate as the float64 loop unless the entries lie well below their block's bound.
+// 2^-54 for the rounding of a float64 operation at that size.
+//
+// What shares an exponent is therefore a row of the left operand and a column of the right one (the
+// entries of one sum), never a block of rows or columns of different size: a row 1e10 times smaller than its
+// neighbour keeps its 56 bits.  A factor common to a column of the left operand, as in P T with
+// T = B (B G B)^{-1/2}, is taken out of it and put into the row of the right one first (a power of two).
+// Only the operands that are bounded alike throughout, the orthonormal U and V in sums over their rows, have
+// one exponent per 64 rows.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -27,11 +33,18 @@ namespace fx {
 
 constexpr int kTerms = 64;
 constexpr int kBad = 1 << 16;  // exponent of a block with a non-finite entry: its products become NaN
+constexpr int kZero = -4096;   // exponent of zeros where exponents are added (below every sum of two others)
 
 // Exponent e with |x| < 2^e, from the upper word of the largest |x| (zero and subnormal: -1022).
 __host__ __device__ inline int exponent(int hi_word) {
   const int ex = (hi_word & 0x7fffffff) >> 20;
   return ex == 0x7ff ? kBad : ex - 1022;
+}
+
+// The same for one finite value, with kZero for zero (and what is below 2^-1042).
+__host__ __device__ inline int value_exponent(int hi_word) {
+  const int h = hi_word & 0x7fffffff;
+  return h ? (h >> 20) - 1022 : kZero;
 }
 
 // x in the fixed point of exponent e (|x| < 2^e, rounded to nearest): .x = hi, .y = lo.

@@ -59,7 +59,6 @@ void iteration(const Shape& s, Buffers& b, bool fp64, bool first, cudaStream_t s
   NA_CUDA(launch_sweep(s, b, fp64, u_new, st));
   NA_CUDA(launch_iter_end(s, b, fp64, st));
   NA_CUDA(launch_gram_p(s, b, fp64, true, st, fp64 && !b.plain ? b.U[u_new] : nullptr, fp64 && !b.plain ? b.B : nullptr));
-  b.d_plain = b.plain;
   b.u_cur = u_new;
   std::swap(b.Y[0], b.Y[1]);
 }

@@ -112,7 +112,7 @@ struct Buffers {
   int64_t ldy;          // leading dimension of Y[] and D: n, rounded up to 4 on the SIMT mixed path
                         // (16-byte aligned rows for its vector and cp.async accesses)
   void* Y[2];           // multiplier ping-pong, m x ldy, TC
-  void* D;              // Delta = X_{k+1} - L_{k+1}, m x ldy, TC (float64 path: fixed point, fix64.cuh)
+  void* D;              // Delta = X_{k+1} - L_{k+1}, m x ldy, TC
   void* P;              // m x rp, TC: X_k V_k
   void* U[2];           // m x rp, TC: U_bar ping-pong
   void* W;              // n x rp, TC: X_k^T U_bar
@@ -133,13 +133,12 @@ struct Buffers {
   double* TCm;          // rp x rp : C = W T_C
   float* Qeig_u;        // rp x rp : last U-side eigenvectors (warm start)
   float* Qeig_v;        // rp x rp : last V-side eigenvectors
-  int* ex;              // float64 path: exponents of the fixed-point tiles of U, C and V (64 rows each)
+  int* ex;              // float64 path: exponents of the fixed-point tiles of U and V (64 rows each)
   DevState* st;
   int u_cur;            // which U buffer holds the current U_bar (host-side bookkeeping)
   bool tc;              // tensor-core path (mixed precision, r <= 64, bfloat16 M)
   bool plain;           // float64 path: this iteration's products are float64 loops (kPlainIters; Algorithm 4 always:
                         // its two passes over M bound it, and it starts with cold projector calls)
-  bool d_plain;         // D holds float64 values (the last sweep was a plain one)
   bool full;            // Algorithm 4 on a fixed M: no multiplier or Delta buffers; the
                         // tensor-core path keeps two-term bfloat16 splits of U^T and V^T
   TcBuffers t;          // its extra buffers (Y[] above alias t.Y[] when tc)
@@ -148,14 +147,14 @@ struct Buffers {
 // ---- kernel launchers (sweep.cu / rxr.cu / f64.cu) ----
 // Each launcher returns the cudaError_t of its launch.
 
-// Float64 path (f64.cu), behind the launchers of the same names below.  Between apply_v and the
-// next gram_p, P holds U_bar in fixed point, W holds V_bar and the first W partial holds C.
+// Float64 path (f64.cu), behind the launchers of the same names below.  From apply_u to the next gram_p P holds
+// U_bar in fixed point, and from apply_v to the next wfinal W holds V_bar.
 cudaError_t f64_gram(const Shape& s, const double* parts, int nparts, int64_t part_stride, double* out, int64_t rows,
                      int ctas, const double* A, const double* H, double* gpart, const DevState* dst, cudaStream_t st);
 cudaError_t f64_transform(const Shape& s, const double* src, int64_t rows, int ctas, const double* T, double* dst,
-                          const double* T2, double* dst2, const double* old, double* hpart, void* F, int* eF, void* F2,
-                          int* eF2, const DevState* dstate, cudaStream_t st);
-cudaError_t f64_sweep(const Shape& s, const Buffers& b, cudaStream_t st);
+                          const double* T2, double* dst2, const double* old, double* hpart, void* F, int* eF,
+                          const DevState* dstate, cudaStream_t st);
+cudaError_t f64_sweep(const Shape& s, const Buffers& b, int u_cur, cudaStream_t st);
 cudaError_t f64_wpass(const Shape& s, const Buffers& b, cudaStream_t st);
 
 cudaError_t launch_norm_m(const Shape& s, const Buffers& b, cudaStream_t st);

@@ -193,7 +193,7 @@ size_t carve(const Shape& s, bool fp64, void* base, Buffers* b, bool tc, bool fu
   x.Gsum = static_cast<double*>(c.take(8 * rpsq));
   // (the float64 sweep writes one residual partial per CTA)
   x.resid_part = static_cast<double*>(c.take(8 * (fp64 && !full ? (size_t)s.sweep_grid_x * s.nsplit : (size_t)s.resid_parts)));
-  if (fp64 && !full) x.ex = static_cast<int*>(c.take(4 * ((s.m + 63) / 64 + 2 * ((s.n + 63) / 64))));
+  if (fp64 && !full) x.ex = static_cast<int*>(c.take(4 * ((s.m + 63) / 64 + (s.n + 63) / 64)));
   x.normm_part = static_cast<double*>(c.take(8 * 1024));
   x.B = static_cast<double*>(c.take(8 * rpsq));
   x.Bprev = static_cast<double*>(c.take(8 * rpsq));
@@ -488,7 +488,6 @@ struct Solver {
     // P = sum of partials (float64: of Delta V_bar, + U_bar B_bar, as on the tensor-core path), G_P
     SFR_CUDA(launch_gram_p(s, b, fp64, true, st, fp64 && !b.plain ? b.U[u_new] : nullptr,
                            fp64 && !b.plain ? b.B : nullptr));
-    b.d_plain = b.plain;
     kernels += (first ? 11 : 12) + (s.nchunk >= 32 ? 1 : 0);  // as on the tensor-core path below (+ W pre-sum)
     b.u_cur = u_new;
     std::swap(b.Y[0], b.Y[1]);

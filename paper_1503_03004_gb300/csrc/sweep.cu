@@ -1980,7 +1980,7 @@ cudaError_t launch_apply_u(const Shape& s, const Buffers& b, bool fp64, bool fir
   if (fp64)
     return f64_transform(s, static_cast<const double*>(b.P), s.m, s.gp_blocks, b.TU, static_cast<double*>(b.U[u_new]),
                          nullptr, nullptr, first ? nullptr : static_cast<const double*>(b.U[u_old]),
-                         first ? nullptr : b.Hpart, b.P, b.ex, nullptr, nullptr, b.st, st);
+                         first ? nullptr : b.Hpart, b.P, b.ex, b.st, st);
   if (g_recorder && s.rp <= 32)
     return launch_k<&row_transform_any, 256>(s.gp_blocks, 256, transform_smem<float, 32>(), st, s.rp,
         static_cast<const float*>(b.P), s.m, b.TU, static_cast<float*>(b.U[u_new]), (const double*)nullptr, (float*)nullptr,
@@ -2058,7 +2058,7 @@ cudaError_t launch_wpass(const Shape& s, const Buffers& b, bool fp64, bool first
       if constexpr (std::is_same<TC, double>::value && RP < 32) {
         return f64_wpass(s, b, st);
       } else {
-        if (std::is_same<TC, double>::value && !b.d_plain) return f64_wpass(s, b, st);
+        if (std::is_same<TC, double>::value && !b.plain) return f64_wpass(s, b, st);
         if constexpr (std::is_same<TC, float>::value && RP == 64) {
           if (s.n % 4 == 0 && !b.tc)
             return launch_k<&wpass_mxp_body<float, 64>, 256>(grid, 256, wxp_smem<float, 64>(), st,
@@ -2086,7 +2086,7 @@ cudaError_t launch_wfinal(const Shape& s, const Buffers& b, bool fp64, bool firs
   const double* H = b.Hpart + (size_t)s.gp_blocks * s.rp * s.rp;
   // many row chunks over few columns (tall M): sum the chunks' partials into the first one
   // with a wide reduction first, so the thin kernel does not add hundreds of them per element
-  int nparts = fp64 && !first && !b.d_plain ? s.nchunk64 : s.nchunk;
+  int nparts = fp64 && !first && !b.plain ? s.nchunk64 : s.nchunk;
   if (nparts >= 32) {
     const int64_t len = s.n * s.rp;
     cudaError_t e = by_prec(fp64, [&](auto tc) {
@@ -2135,10 +2135,9 @@ cudaError_t launch_apply_v(const Shape& s, const Buffers& b, bool fp64, cudaStre
           (int64_t)0, 0);
     });
   if (fp64) {
-    const int64_t tu = (s.m + kGramRows - 1) / kGramRows, tv = (s.n + kGramRows - 1) / kGramRows;
+    const int64_t tu = (s.m + kGramRows - 1) / kGramRows;
     return f64_transform(s, static_cast<const double*>(b.W), s.n, s.gw_blocks, b.TV, static_cast<double*>(b.V), b.TCm,
-                         static_cast<double*>(b.C), nullptr, nullptr, b.W, b.ex + tu + tv, b.Wpart, b.ex + tu,
-                         b.st, st);
+                         static_cast<double*>(b.C), nullptr, nullptr, b.W, b.ex + tu, b.st, st);
   }
   if (g_recorder && s.rp <= 32)
     return launch_k<&row_transform_any, 256>(s.gw_blocks, 256, transform_smem<float, 32>(), st, s.rp,
@@ -2210,7 +2209,7 @@ static cudaError_t launch_sweep_mx(const Shape& s, const Buffers& b, int u_cur, 
 cudaError_t launch_sweep(const Shape& s, const Buffers& b, bool fp64, int u_cur, cudaStream_t st) {
   // Y ping-pong: iteration k (0-based count of completed iterations) reads Y[k % 2] and writes
   // Y[(k + 1) % 2].  The host tracks k because graphs are replayed per iteration parity.
-  if (fp64 && !b.plain) return f64_sweep(s, b, st);
+  if (fp64 && !b.plain) return f64_sweep(s, b, u_cur, st);
   if (mx_path(s, fp64) || mx64(s, b, fp64)) return launch_sweep_mx(s, b, u_cur, st);
   // mixed precision above rank 32 outside the tensor-core path, and the plain float64 iterations
   dim3 grid(s.sweep_grid_x, s.nsplit);

@@ -50,3 +50,31 @@ def test_truncated_svd_rows_of_different_size(ctx, r):
     sol = B.opt_full_torch(ctx, torch.from_numpy(M).cuda(), r, tol=0.0, max_iter=12, precision=B.PREC_FP64)
     L = (sol.U @ sol.B @ sol.V.T).cpu().numpy()
     assert _row_error(L, Ur @ Br @ Vr.T) <= ROW_TOL
+
+
+def _planted(m, n, r, seed):
+    """Low rank with independent first r columns, plus outliers of five times the entries' size on 5 % of them."""
+    rng = np.random.default_rng(seed)
+    R = rng.standard_normal((r, n))
+    R[:, :r] = np.sqrt(r) * np.linalg.qr(R[:, :r])[0]
+    S = np.where(rng.random((m, n)) < 0.05, rng.uniform(-5, 5, (m, n)) * np.sqrt(r), 0.0)
+    return rng.standard_normal((m, r)) @ R + S
+
+
+# The path's own bar (1e-9 in norm), here for each row or column in its own size.
+@pytest.mark.parametrize("m,n,r", [(333, 260, 5), (300, 321, 12), (400, 260, 24), (390, 330, 50), (2100, 96, 8)])
+def test_robust_rows_of_different_size(ctx, m, n, r):
+    M = _scales(m, r)[:, None] * _planted(m, n, r, 10 + r)
+    ref = O.fr_adm(M, r, rho=1.5, mu0=0.1, fixed_iters=12)
+    sol = B.solve_torch(ctx, torch.from_numpy(M).cuda(), r, fixed_iters=12, rho=1.5, mu0=0.1)
+    assert _row_error((sol.U @ sol.B @ sol.V.T).cpu().numpy(), ref.L) <= 1e-9
+
+
+@pytest.mark.parametrize("m,n,r", [(260, 333, 5), (321, 300, 12), (260, 400, 24), (330, 390, 50), (96, 2100, 8)])
+def test_robust_columns_of_different_size(ctx, m, n, r):
+    s = _scales(n, r)
+    s[:r] = 1.0  # (the iteration starts from the first r columns)
+    M = s[None, :] * _planted(m, n, r, 10 + r)
+    ref = O.fr_adm(M, r, rho=1.5, mu0=0.1, fixed_iters=12)
+    sol = B.solve_torch(ctx, torch.from_numpy(M).cuda(), r, fixed_iters=12, rho=1.5, mu0=0.1)
+    assert _row_error((sol.U @ sol.B @ sol.V.T).cpu().numpy().T, ref.L.T) <= 1e-9
