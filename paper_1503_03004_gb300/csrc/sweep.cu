@@ -1271,6 +1271,15 @@ __device__ __forceinline__ void sweep_mxp_body(const VGrid& vg__, const TMs* __r
     const int jn = cols;
     const float* x0p = ys + 2 * tr * ldx;
     const float* vp = Vs + QA * tc;
+    // above rank 32 a tile's sum is formed by itself and then added: with one chain over all columns of a split (and all rows
+    // of a chunk in the W pass) L was off by 9.9e-6 instead of 1.4e-6 at 40000 x 4096, r = 40; 72.8 -> 73.8 us a sweep
+    // at 2048 x 2048, r = 40
+    float qt[2][QA];
+    if constexpr (RP == 64) {
+#pragma unroll
+      for (int c = 0; c < QA; ++c) qt[0][c] = qt[1][c] = 0.f;
+    }
+    float(&qa)[2][QA] = RP == 64 ? qt : q;
 #pragma unroll 2
     for (int jj = 0; jj < jn; jj += 4) {
       const float4 w0 = *reinterpret_cast<const float4*>(x0p + jj), w1 = *reinterpret_cast<const float4*>(x0p + ldx + jj);
@@ -1293,10 +1302,14 @@ __device__ __forceinline__ void sweep_mxp_body(const VGrid& vg__, const TMs* __r
         }
 #pragma unroll
         for (int c = 0; c < QA; ++c) {
-          q[0][c] = fmaf(x0[s4], v[c], q[0][c]);
-          q[1][c] = fmaf(x1[s4], v[c], q[1][c]);
+          qa[0][c] = fmaf(x0[s4], v[c], qa[0][c]);
+          qa[1][c] = fmaf(x1[s4], v[c], qa[1][c]);
         }
       }
+    }
+    if constexpr (RP == 64) {
+#pragma unroll
+      for (int c = 0; c < QA; ++c) q[0][c] += qt[0][c], q[1][c] += qt[1][c];
     }
     if (last) {  // row block done: its Q partial and residual
 #pragma unroll
@@ -1468,6 +1481,16 @@ __device__ __forceinline__ void wpass_mxp_body(const VGrid& vg__, const TS* __re
     __syncthreads();
     const TS* xs = Xs + (k % kWxStages) * XS;
     const float* us = Us + (k % kWxStages) * US;
+    // (with one row group a tile's sum is formed by itself and then added, as in sweep_mxp_body: 275 -> 289 us at 8192 x 8192,
+    // r = 64)
+    float tile[4][4];
+    if constexpr (RS == 1) {
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) tile[x][c] = 0.f;
+    }
+    float(&ta)[4][4] = RS == 1 ? tile : acc;
 #pragma unroll 4
     for (int ii = rg; ii < BR; ii += RS) {
       float xv[4];
@@ -1484,7 +1507,13 @@ __device__ __forceinline__ void wpass_mxp_body(const VGrid& vg__, const TS* __re
 #pragma unroll
       for (int x = 0; x < 4; ++x)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[x][c] = fmaf(xv[x], uv[c], acc[x][c]);
+        for (int c = 0; c < 4; ++c) ta[x][c] = fmaf(xv[x], uv[c], ta[x][c]);
+    }
+    if constexpr (RS == 1) {
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[x][c] += tile[x][c];
     }
     __syncthreads();  // stage k % stages is refilled by the next iteration's issue
   }
