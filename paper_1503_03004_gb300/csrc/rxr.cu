@@ -272,7 +272,7 @@ template <int RP> struct RxrSmem {  // 214 KB at RP = 64
   float F1[RP * LD];    // scratch
   float F2[RP * LD];    // scratch
   float lam[64], sq[64], isq[64];  // (all 64 read as two values per lane; entries past r unused)
-  double red[32];
+  double red[64];
   unsigned mx[16];      // block-wide maxima, one slot each (bits of non-negative floats)
   float cs[RP / 2], sn[RP / 2];
   int pp[RP / 2], qq[RP / 2];
@@ -308,18 +308,6 @@ __device__ __forceinline__ float block_max_f(float v, unsigned* slot) {
   if ((threadIdx.x & 31) == 0) atomicMax(slot, m);
   __syncthreads();
   return __uint_as_float(*slot);
-}
-
-// Block-wide sum of floats (it steers decisions only).
-template <int NT> __device__ __noinline__ float block_sum_f(float v, float* red) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0) red[w] = v;
-  __syncthreads();
-  float t = l < NT / 32 ? red[l] : 0.f;
-  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  __syncthreads();
-  return t;
 }
 
 // Sum of x[0 .. r), r <= 64, by every warp for itself.
@@ -367,14 +355,20 @@ __device__ __noinline__ void jacobi_f32(float* A, float* Q, int n2, int max_swee
   const bool pow2 = (np & (np - 1)) == 0;
   const int lg = 31 - __clz(np);
   for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    float off = 0.f, dia = 0.f;
-    for (int e = threadIdx.x; e < n2 * n2; e += blockDim.x) {
-      const int i = e / n2, j = e % n2;
-      const float v = A[i * LD + j];
-      if (i == j) dia = fmaf(v, v, dia); else off = fmaf(v, v, off);
+    // (summed by rows, a warp each, then over the rows by every warp: the sums decide how many sweeps run, so their order
+    // must not depend on the number of threads, which differs between the kernels a rank may run in)
+    const int lane_ = threadIdx.x & 31;
+    float* rows = reinterpret_cast<float*>(red);  // [64] off-diagonal, [64] diagonal squares
+    for (int i = threadIdx.x >> 5; i < n2; i += kThreads / 32) {
+      const float a = lane_ < n2 ? A[i * LD + lane_] : 0.f, b = lane_ + 32 < n2 ? A[i * LD + lane_ + 32] : 0.f;
+      float v = lane_ == i ? 0.f : a * a;
+      if (lane_ + 32 != i) v = fmaf(b, b, v);
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane_ == 0) rows[i] = v;
+      if (lane_ == (i & 31)) rows[64 + i] = i < 32 ? a * a : b * b;
     }
-    off = block_sum_f<kThreads>(off, reinterpret_cast<float*>(red));
-    dia = block_sum_f<kThreads>(dia, reinterpret_cast<float*>(red));
+    __syncthreads();
+    const float off = warp_sum64(rows, 1, n2), dia = warp_sum64(rows + 64, 1, n2);
     // off-diagonal mass below (1e-3)^2 of the diagonal: each float64 Newton step that follows
     // contracts the residual by about this factor (the next call refines the basis further)
     if (!(off > 1e-6 * dia)) break;
