@@ -352,7 +352,7 @@ struct Solver {
   int graph_kernels = 0;
   TcMaps maps;          // tensor maps of the current tensor-core solve (captured by value in graphs)
   bool last_tc = false; // whether the last solve took the tensor-core path
-  // profiling: kernel counters and events (slot 0: eager iteration, slots 1-2: the graph's two)
+  // profiling: kernel counters and events (slots as for ev below)
   bool profile = false;
   bool profile_pass_only = false;  // time only the m x n pass (sweep or P pass), not W pass / r x r
   bool count_stats = false;
@@ -363,7 +363,9 @@ struct Solver {
   double bytes[SFR_STAT_COUNT] = {};
   double sweep_bytes = 0, wpass_bytes = 0, wpass_first_bytes = 0;  // per launch, set per solve
   int pass_kind = SFR_STAT_SWEEP;  // class of the m x n pass timed in event slot 0 (sweep or P pass)
-  cudaEvent_t ev[5][4][2] = {};       // slot 0: eager iteration; 1-2: graph A; 3-4: graph B
+  // slot 0: iteration 1; 1-2: graph A; 3-4: graph B; 5 and on: the eager iterations after the first
+  static constexpr int kEagerSlot = 5;
+  cudaEvent_t ev[kEagerSlot + kPlainIters][4][2] = {};
   cudaEvent_t done_ev[2] = {};        // completion of the last launch of graph A / B
   DevState* host_state2 = nullptr;    // pinned state copies taken after graph A / B
   std::unique_ptr<Solver> aux;        // FR-Nys: solves the second block concurrently (own stream)
@@ -417,19 +419,20 @@ struct Solver {
     // inside stream capture an event record becomes a graph node only with the external flag,
     // and that flag is refused outside capture
     const unsigned flags = capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
-    // profile 2: the sweep of the eager first iteration (slot 0) and of the first iteration of
-    // each replay of graph A (slot 1), one iteration in four
-    const bool timed = profile && (!profile_pass_only || (k == 0 && slot <= 1));
+    const bool timed = profile && (!profile_pass_only || (k == 0 && pass_slot(slot)));
     if (timed) SFR_CUDA(cudaEventRecordWithFlags(ev[slot][k][0], on, flags));
     SFR_CUDA(f());
     if (timed) SFR_CUDA(cudaEventRecordWithFlags(ev[slot][k][1], on, flags));
   }
 
+  // profile 2: one iteration in four, the eager ones 1 and 5 and the first of each replay of graph A
+  static bool pass_slot(int slot) { return slot <= 1 || slot == kEagerSlot + 3; }
+
   // Accumulate the event durations of the iterations that ran in `slot`s [first, first + count).
   void harvest(int first, int count) {
     if (!profile || !count_stats) return;
     for (int sl = first; sl < first + count; ++sl) {
-      if (profile_pass_only && sl > 1) break;  // see timed_launch_on
+      if (profile_pass_only && !pass_slot(sl)) continue;
       float ms;
       SFR_CUDA(cudaEventElapsedTime(&ms, ev[sl][0][0], ev[sl][0][1]));
       total_ms[pass_kind] += ms;
@@ -585,7 +588,8 @@ struct Solver {
     make_done_events();
     SFR_CUDA(cudaMemcpyAsync(host_state, after_first.st, sizeof(DevState), cudaMemcpyDeviceToHost, stream));
     SFR_CUDA(cudaStreamSynchronize(stream));
-    if (timed_first) harvest(0, host_state->iter >= 1 ? 1 : 0);
+    if (timed_first) harvest(0, std::min(host_state->iter, 1));
+    harvest(kEagerSlot, std::max(std::min(host_state->iter, eager) - 1, 0));
     int launched = eager, last_iter = host_state->iter, which = 0;
     int queue[2], queued = 0;  // launched graphs whose state has not been read yet (oldest first)
     bool stop = host_state->done != 0;
@@ -693,7 +697,7 @@ struct Solver {
     const int eager = plain_start(s.rp, fp64) ? kPlainIters + 1 : 1;
     for (int k = 0; k < eager; ++k) {
       b.plain = eager > 1 && k < kPlainIters;
-      count(SFR_STAT_ALL, enqueue_iteration(s, b, fp64, k == 0, 0));
+      count(SFR_STAT_ALL, enqueue_iteration(s, b, fp64, k == 0, k ? kEagerSlot + k - 1 : 0));
     }
     count(SFR_STAT_SWEEP, eager);
     count(SFR_STAT_WPASS, eager);
