@@ -693,12 +693,13 @@ struct Solver {
     if (!tc && mx_path(s, fp64)) tune_mx(s, b, p.m_dtype);
 
     // iteration 1 (X_1 = M, V_1 = I_{n x r}), eager; with a plain start (kPlainIters) also the plain
-    // iterations and the first one after them
-    const int eager = plain_start(s.rp, fp64) ? kPlainIters + 1 : 1;
+    // iterations and the first one after them, or as many as the solve may run (made odd)
+    const int eager = plain_start(s.rp, fp64) ? std::min(kPlainIters + 1, h.max_iter | 1) : 1;
     for (int k = 0; k < eager; ++k) {
-      b.plain = eager > 1 && k < kPlainIters;
+      b.plain = plain_start(s.rp, fp64) && k < kPlainIters;
       count(SFR_STAT_ALL, enqueue_iteration(s, b, fp64, k == 0, k ? kEagerSlot + k - 1 : 0));
     }
+    b.plain = false;  // (the graphs, captured from here, run the fixed-point kernels)
     count(SFR_STAT_SWEEP, eager);
     count(SFR_STAT_WPASS, eager);
     count(SFR_STAT_RXR, 2 * eager);
