@@ -359,14 +359,24 @@ __device__ __noinline__ void jacobi_f32(float* A, float* Q, int n2, int max_swee
     // must not depend on the number of threads, which differs between the kernels a rank may run in)
     const int lane_ = threadIdx.x & 31;
     float* rows = reinterpret_cast<float*>(red);  // [64] off-diagonal, [64] diagonal squares
-    for (int i = threadIdx.x >> 5; i < n2; i += kThreads / 32) {
-      const float a = lane_ < n2 ? A[i * LD + lane_] : 0.f, b = lane_ + 32 < n2 ? A[i * LD + lane_ + 32] : 0.f;
-      float v = lane_ == i ? 0.f : a * a;
-      if (lane_ + 32 != i) v = fmaf(b, b, v);
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane_ == 0) rows[i] = v;
-      if (lane_ == (i & 31)) rows[64 + i] = i < 32 ? a * a : b * b;
+    constexpr int NW_ = kThreads / 32, RPW = RPMAX / NW_;  // rows of a warp: their sums are taken side by side
+    float v_[RPW];
+#pragma unroll
+    for (int u = 0; u < RPW; ++u) {
+      const int i = (int)(threadIdx.x >> 5) + NW_ * u;
+      const bool in = i < n2;
+      const float a = in && lane_ < n2 ? A[i * LD + lane_] : 0.f;
+      const float b = RPMAX > 32 && in && lane_ + 32 < n2 ? A[i * LD + lane_ + 32] : 0.f;
+      v_[u] = lane_ == i ? 0.f : a * a;
+      if (RPMAX > 32 && lane_ + 32 != i) v_[u] = fmaf(b, b, v_[u]);
+      if (in && lane_ == (i & 31)) rows[64 + i] = i < 32 ? a * a : b * b;
     }
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int u = 0; u < RPW; ++u) v_[u] += __shfl_xor_sync(0xffffffffu, v_[u], o);
+#pragma unroll
+    for (int u = 0; u < RPW; ++u)
+      if (lane_ == 0 && (int)(threadIdx.x >> 5) + NW_ * u < n2) rows[(threadIdx.x >> 5) + NW_ * u] = v_[u];
     __syncthreads();
     const float off = warp_sum64(rows, 1, n2), dia = warp_sum64(rows + 64, 1, n2);
     // off-diagonal mass below (1e-3)^2 of the diagonal: each float64 Newton step that follows
