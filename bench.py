@@ -570,7 +570,8 @@ def run_config(args):
     hbm, src = peaks()
     avg = sw["total_ms"] / max(1, sw["timed"])
     if prec == B.PREC_FP64:
-        # float64 sweep: L rebuild (2 r) and (L + Delta) V (2 r) flops per element of the sweep
+        # float64 sweep: L rebuild (2 r) and Delta V (2 r) flops per element; above rank 16 the average holds the six
+        # sweeps of the plain start, which run on the float64 units
         achieved = 4 * r * m * n / (avg * 1e-3) / 1e12
         roof = {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                 "frac": achieved / FP64_PEAK_TFLOPS, "traffic": None, "kernel": "fused sweep (float64 as fixed point)",

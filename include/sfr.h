@@ -58,7 +58,10 @@ typedef enum { SFR_F64 = 0, SFR_F32 = 1, SFR_BF16 = 2 } sfr_dtype;
 
 /* Arithmetic of the m x n sweep.  The r x r projectors and the convergence
  * test are float64 in both modes.
- *   SFR_PREC_FP64:  float64 everywhere (M may be stored f64, f32 or bf16).
+ *   SFR_PREC_FP64:  float64 storage and arithmetic (M may be stored f64, f32 or bf16); the
+ *                   products of FR-ADM are summed exactly in fixed point, each row of a left
+ *                   operand and column of a right one with 56 bits below its largest entry,
+ *                   which rounds no more than float64 multiply-add does.
  *   SFR_PREC_MIXED: float32 sweep arithmetic and multiplier storage, float64
  *                   factors and r x r steps. */
 typedef enum { SFR_PREC_FP64 = 0, SFR_PREC_MIXED = 1 } sfr_precision;

@@ -1,8 +1,9 @@
 // Float64 path: the m x n passes and the thin (m x r, n x r) kernels, with every inner product in
 // fixed point on the integer units (fix64.cuh).  A float64 FMA loop over the same products ran at
 // GB300's 1.2 TFLOP/s: at 4096 x 4096, r = 64 the sweep took 3.95 ms, the W pass 2.4 ms and the thin
-// kernels 0.8 ms of a 7.3 ms iteration.  Element-wise float64 arithmetic (about eight operations per
-// element of M) stays on the float64 units and now bounds the sweep for r below about 40.
+// kernels 0.8 ms of a 7.3 ms iteration; now 1.21, 0.66 and 0.24 of 2.35 ms.  Element-wise float64 arithmetic (about eight
+// operations per element of M) stays on the float64 units and bounds the sweep at small r: ncu, 4096 x 4096, float64
+// pipe 64 % and wide-multiply pipe 33 % active at r = 10, 36 % and 66 % at r = 64 (W pass 19 % and 68 %).
 //
 // Exponents (fix64.cuh): the thin kernels and the sweep convert their operands themselves, each row of P, U, C and W
 // and each column of an r x r factor or of a Gram operand with its own exponent; Delta is held in float64, and has

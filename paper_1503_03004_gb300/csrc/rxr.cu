@@ -30,8 +30,9 @@
 // latency rather than arithmetic.  It is therefore built per padded rank (Dim): r <= 8 runs in one
 // warp, r <= 16 in one CTA of 128 threads, r <= 32 in clusters of 256-thread CTAs, r <= 64 in clusters of 512,
 // element-wise steps are done where a product's results are stored (Epi), and the statistics of the r
-// eigenvalue estimates are taken by every warp for itself.  A warm call (mixed path) before -> now: r = 3 31 -> 16,
-// r = 32 38 -> 32 r = 48 52 -> 48, r = 64 95 -> us, with the same results to the last bit.
+// eigenvalue estimates are taken by every warp for itself.  The mean call of a solve of 60 iterations (1536 x 1024, mixed path,
+// partial sums included), one kernel of 512 threads for every rank -> now: r = 3 29.8 -> 20.6 us, r = 10 35.7 -> 25.7,
+// r = 32 52.1 -> 43.8, r = 38 65.1 -> 63.6, r = 48 82.3 -> 78.1, r = 64 101.3 -> 89.4.
 #include <cooperative_groups.h>
 
 #include <type_traits>
@@ -100,8 +101,8 @@ __device__ __noinline__ void mm_dist(const double* A, const TB* B, TCo* C, int r
   cg::cluster_group cl = cg::this_cluster();
   const int cs = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int rpc = (r + cs - 1) / cs, i0 = min(r, rank * rpc), i1 = min(r, i0 + rpc);
-  // (packed in r, not RP: a warp with idle lanes takes the float64 pipe as long as a full one:
-  // r = 5 23.6 -> 21.7 us a call, r = 10 34.5 -> 31.7)
+  // (packed in r, not RP: a warp with idle lanes takes the float64 pipe as long as a full one: the kernel alone on
+  // the float64 path, r = 5 23.6 -> 21.7 us, r = 10 34.5 -> 31.7)
   for (int e = threadIdx.x; e < (i1 - i0) * r; e += DM::NT) {
     const int i = i0 + e / r, j = e % r;
     // four independent chains (k mod 4) keep the float64 pipe busy with few warps per SM

@@ -1030,10 +1030,10 @@ template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile(
 // its 4-column groups XORed with the rank group, so that neither the 4-byte copies nor the 16-byte reads meet in a
 // bank) and U of the next pair while Q is.  So C, U and V need one buffer each (with one column tile per row block:
 // two of U, copied with Y), which leaves room for a third CTA per SM on narrow matrices and a second one above rank
-// 32.  X = L + Delta overwrites the Y tile; the threads' residuals stand in its padding.
+// 32 (float32 M: up to rank 48).  X = L + Delta overwrites the Y tile; the threads' residuals stand in its padding.
 // A thread's columns are 4 tc .. + 3 and 32 + 4 tc .. + 3, so that 8 threads read 128 contiguous bytes; sums over
 // ranks and columns run in order, 4 at a time from 16-byte reads (zeros past r and past the last column add nothing).
-// The kernel is bound by issue (60 % of the slots) and by the latency of its shared-memory reads, hence also: addresses
+// The kernel is bound by issue (55 to 57 % of the slots, ncu) and by the latency of its shared-memory reads, hence also: addresses
 // step from one base per tile, limits are 32-bit, and masks are left out where zeros do the same.
 // Per sweep: 4096 x 2048, r = 32, bfloat16 57 us (61 with masks and 64-bit addresses, 105 with plain loads of C and V
 // after the barrier); 2^20 x 40, r = 3, float32 133 us (186 with two CTAs per SM in four stages); 2048 x 2048, r = 40,
