@@ -50,6 +50,10 @@ template <int RP_> struct Dim {
   static constexpr int RP = RP_, NT = RP == 64 ? 512 : RP == 32 ? 256 : RP == 16 ? 128 : 32;
   static constexpr int TM = RP == 64 ? 4 : RP == 32 ? 2 : 1, TN = RP == 64 ? 4 : 2;
   static constexpr int LD = RP + 4, LDD = RP;
+  // One CTA per SM is all that is asked for: without that the registers of the functions the kernel calls were held to
+  // 72 or 80, and the body kept its own on the stack around every call (grouped, padded rank 32: 88 bytes; with it 112 to
+  // 140 registers and none).  FR-Nys 7805 x 7805, r = 21 10.6 -> 9.7 ms, 4096 x 2048, r = 32 from the host 10.2 -> 9.7.
+  static constexpr int kBounds = per_sm(NT, 1);
 };
 
 __device__ __forceinline__ bool stopped(const DevState* st) { return *(volatile const int32_t*)&st->done != 0; }
@@ -985,9 +989,9 @@ static int rxr_cluster_size() {
   static const int best = [] {
     constexpr size_t smem = sizeof(RxrSmem<RP>);
     constexpr int NT = Dim<RP>::NT;
-    auto kern = body_kernel_of<&rxr_body<RP>, NT>();
+    auto kern = body_kernel_of<&rxr_body<RP>, Dim<RP>::kBounds>();
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) cudaGetLastError();
-    if (set_smem_attr<body_kernel_of<&rxr_body<RP>, NT>()>(smem) != cudaSuccess) cudaGetLastError();
+    if (set_smem_attr<body_kernel_of<&rxr_body<RP>, Dim<RP>::kBounds>()>(smem) != cudaSuccess) cudaGetLastError();
     for (int cs : {16, 8}) {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(cs);
@@ -1019,7 +1023,7 @@ cudaError_t launch_rxr(const Shape& s, const Buffers& b, bool v_side, cudaStream
   // settles, so the V side's first-order refinement holds from the fourth iteration on)
   auto go = [&](auto rpc) {
     constexpr int RP = decltype(rpc)::value, NT = Dim<RP>::NT;
-    return launch_k_cluster<&rxr_body<RP>, NT>(rxr_cluster_size<RP>(), NT, sizeof(RxrSmem<RP>), st, (const double*)b.Gsum,
+    return launch_k_cluster<&rxr_body<RP>, Dim<RP>::kBounds>(rxr_cluster_size<RP>(), NT, sizeof(RxrSmem<RP>), st, (const double*)b.Gsum,
                                               s.rp, s.r, b.B, v_side ? b.TV : b.TU, v_side ? b.TCm : (double*)nullptr,
                                               (const float*)b.Qeig_u, v_side ? b.Qeig_v : b.Qeig_u, v_side ? 1 : 0,
                                               fp64 ? 0 : 1, b.st);
