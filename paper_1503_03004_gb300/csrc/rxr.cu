@@ -31,8 +31,8 @@
 // warp, r <= 16 in one CTA of 128 threads, r <= 32 in clusters of 256-thread CTAs, r <= 64 in clusters of 512,
 // element-wise steps are done where a product's results are stored (Epi), and the statistics of the r
 // eigenvalue estimates are taken by every warp for itself.  The mean call of a solve of 60 iterations (1536 x 1024, mixed path,
-// partial sums included), one kernel of 512 threads for every rank -> now: r = 3 29.8 -> 20.6 us, r = 10 35.7 -> 25.7,
-// r = 32 52.1 -> 43.8, r = 38 65.1 -> 63.6, r = 48 82.3 -> 78.1, r = 64 101.3 -> 89.4.
+// partial sums included), one kernel of 512 threads for every rank -> now: r = 3 29.8 -> 20.6 us, r = 10 35.7 -> 24.2,
+// r = 32 52.1 -> 40.4, r = 38 65.1 -> 63.2, r = 48 82.3 -> 77.4, r = 64 101.3 -> 89.7.
 #include <cooperative_groups.h>
 
 #include <type_traits>
